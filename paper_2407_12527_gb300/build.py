@@ -32,7 +32,10 @@ def nvcc() -> str:
 
 
 def sources():
-    return sorted(CSRC.glob("*.cu"))
+    # the sweeps first: their many template instances take the longest to compile, the
+    # dense operator's one-row sweep longest of all
+    return sorted(CSRC.glob("*.cu"), key=lambda p: (not p.stem.endswith("row_dense"),
+                                                    not p.stem.startswith("sweep"), p.name))
 
 
 def _stale() -> bool:
@@ -60,7 +63,7 @@ def build(force: bool = False, verbose: bool = False) -> Path:
         (BUILD / (src.stem + ".ptxas.txt")).write_text(r.stderr)
         return obj
 
-    with ThreadPoolExecutor(max_workers=min(8, os.cpu_count() or 1)) as ex:
+    with ThreadPoolExecutor(max_workers=min(16, os.cpu_count() or 1)) as ex:
         objs = list(ex.map(compile_one, sources()))
     tmp = OUT.with_suffix(f".so.tmp{os.getpid()}")
     cmd = [nvcc()] + ARCH + ["-shared", "-cudart", "shared", "-o", str(tmp)] + [str(o) for o in objs]

@@ -363,8 +363,19 @@ int source_mode(const rom_ctx *ctx)
     return 0;
 }
 
+// whether the one-row sweep of this layout is the ring-staged kernel (sweep2d_ring.cuh);
+// rows too wide for its shared memory run on sweep2d_row.cuh
+bool ring_sweep(const rom_ctx *ctx)
+{
+    return ctx->dim == 2 &&
+           romk::sweep2d_ring_fits(ctx->I, source_mode(ctx), ctx->homog && !batch(ctx));
+}
+
 // rows per wavefront step of the X-Y sweep: forced by the option, else the autotuned
-// value (moment modes), else 4; 1 is the one-row kernel (sweep2d_row.cuh)
+// value (moment modes), else 1 where the ring-staged one-row kernel runs and the work-item
+// size is left to the library (it is the fastest at every size measured: 256 x 256 x 64
+// samples of 16 49 us per sweep against 88 with 4 rows, 100 x 100 x 16 of 36 18 against 62,
+// 256 ordinates of one 256 x 256 sample 35 against 68), else 4
 int choose_rows(const rom_ctx *ctx)
 {
     if (ctx->dim != 2) return 4;
@@ -376,6 +387,7 @@ int choose_rows(const rom_ctx *ctx)
     if (ctx->opt.rows_per_step == 1 || ctx->opt.rows_per_step == 2 || ctx->opt.rows_per_step == 4)
         return ctx->opt.rows_per_step;
     if (ctx->opt.tile_g == -1 && ctx->tuned_h > 0) return ctx->tuned_h;
+    if (ctx->opt.tile_g == 0 && ring_sweep(ctx)) return 1;
     return 4;
 }
 
@@ -390,6 +402,7 @@ int choose_g(const rom_ctx *ctx)
     if (ctx->opt.tile_g == 1 || ctx->opt.tile_g == 2 || ctx->opt.tile_g == 4)
         return std::min(ctx->opt.tile_g, cap);
     if (ctx->opt.tile_g == -1 && ctx->tuned_g > 0) return std::min(ctx->tuned_g, cap);
+    const bool ring = ctx->opt.rows_per_step <= 1 && ring_sweep(ctx);
     // largest G that still gives at least two work items per SM
     for (int G : {4, 2}) {
         if (G > cap) continue;
@@ -397,7 +410,7 @@ int choose_g(const rom_ctx *ctx)
         for (int s = 0; s < ctx->S; ++s) n += 4 * ((ctx->M[s] / 4 + G - 1) / G);
         if (n >= 2LL * ctx->sm_count) return G;
     }
-    return 1;
+    return ring ? 2 : 1;  // (the ring-staged kernel has no one-ordinate form)
 }
 
 // 3D: work items of G = 2 ordinates of one sample and octant (1 with tile_g =
@@ -530,9 +543,19 @@ int build_batch_tables(rom_ctx *ctx)
 int build_items(rom_ctx *ctx)
 {
     if (ctx->dim == 3) return build_items3(ctx);
+    romk::GridDesc one{ctx->I, ctx->J, ctx->NXP, 0.f, 0.f, 0.f, 0.f, 0, (long long)ctx->J * ctx->NXP};
     if (batch(ctx)) {
         int rc = build_batch_tables(ctx);
         if (rc) return rc;
+    } else {  // the one grid's entry (the stream is synchronised below)
+        const double wx = ctx->hi[0] - ctx->lo[0], wy = ctx->hi[1] - ctx->lo[1];
+        one.inv_dx = (float)(ctx->I / wx);
+        one.inv_dy = (float)(ctx->J / wy);
+        one.dx = (float)(wx / ctx->I);
+        one.dy = (float)(wy / ctx->J);
+        int rc = ensure(ctx, ctx->gdesc, sizeof one);
+        if (rc) return rc;
+        CK(cudaMemcpyAsync(ctx->gdesc.p, &one, sizeof one, cudaMemcpyHostToDevice, ctx->stream));
     }
     const int G = choose_g(ctx);
     ctx->G_used = G;
@@ -649,6 +672,7 @@ romk::SweepArgs sweep_args(const rom_ctx *ctx)
         a.grids = (const romk::GridDesc *)ctx->gdesc.p;
         a.soff = (const long long *)ctx->soff_dev.p;
     }
+    a.gdesc = (const romk::GridDesc *)ctx->gdesc.p;
     a.leak = has_balance(ctx) ? (double *)ctx->leak.p : nullptr;
     a.dx = (float)((ctx->hi[0] - ctx->lo[0]) / ctx->I);
     a.dy = (float)((ctx->hi[1] - ctx->lo[1]) / ctx->J);
@@ -828,6 +852,9 @@ cudaError_t launch_xy_sweep(const rom_ctx *ctx, const romk::SweepArgs &sa, int G
 {
     const int L = (ctx->I + romk::kCols - 1) / romk::kCols;
     const int nwarps = (L + 31) / 32;
+    if (H == 1 && ring_sweep(ctx))
+        return romk::launch_sweep2d_ring(sa, (int)ctx->items.size(), G, ctx->opt.scheme,
+                                         ctx->homog && !batch(ctx), ctx->MOM, st);
     if (H == 1) {
         if (batch(ctx))
             return romk::launch_sweep2d_row_batch(sa, (int)ctx->items.size(), nwarps, G,
@@ -974,12 +1001,15 @@ int autotune_g(rom_ctx *ctx)
     const int cap = source_mode(ctx) == 0 ? 2 : 4;
     float best_ms = 0.f;
     int best = 0, best_h = 4, rc;
-    const bool dense = source_mode(ctx) == 0;
+    const bool dense = source_mode(ctx) == 0, ring = ring_sweep(ctx);
     // 0: every H (dense operator mode: 1 and 4; 2 there means 4)
     const int want_h = dense && ctx->opt.rows_per_step == 2 ? 4 : ctx->opt.rows_per_step;
     for (int cand = 0; cand < 9; ++cand) {
         const int G = 1 << (cand / 3), H = 1 << (cand % 3);  // H = 1, 2, 4
         if (G > cap || (want_h != 0 && H != want_h) || (dense && H == 2)) continue;
+        // the ring-staged one-row kernel, where it runs, beats the 2- and 4-row shapes, and
+        // has no one-ordinate form
+        if (ring && (G == 1 || (want_h == 0 && H != 1)) && !(want_h > 1)) continue;
         ctx->opt.tile_g = G;
         if ((rc = build_items(ctx))) return rc;
         if ((rc = ensure_state(ctx))) return rc;  // phi, sources, accumulators

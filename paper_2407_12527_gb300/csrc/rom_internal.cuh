@@ -81,6 +81,7 @@ struct SweepArgs {
     // sizes and coefficient block, and its sample's state starts at soff[sample]
     const GridDesc *grids;      // [grids]
     const long long *soff;      // [S] first float of the sample's [MOM][cells] block
+    const GridDesc *gdesc;      // the same table, or the one grid's entry (sweep2d_ring.cuh)
     // moment modes: the net leakage of each sample's sweep (nullptr: not kept)
     double *leak;               // [S]
     float dx, dy;               // leakage weights |c| dy, |s| dx
@@ -345,6 +346,11 @@ cudaError_t launch_sweep2d_row(const SweepArgs &a, int n_items, int nwarps, int 
                                bool homog, int mom, cudaStream_t st);
 cudaError_t launch_sweep2d_row_batch(const SweepArgs &a, int n_items, int nwarps, int G,
                                      int scheme, int mom, cudaStream_t st);
+// the moment modes with the rows staged through shared memory (sweep2d_ring.cuh), one grid
+// or a batch of them (a.I: the widest); fits: whether a row's rings fit a CTA
+bool sweep2d_ring_fits(int I, int mom, bool homog);
+cudaError_t launch_sweep2d_ring(const SweepArgs &a, int n_items, int G, int scheme, bool homog,
+                                int mom, cudaStream_t st);
 cudaError_t launch_sweep3d(const Sweep3Args &a, int n_ctas, int nwarps, int G, int scheme,
                            cudaStream_t st);
 int sweep3d_ctas_per_sm(int nwarps, int G);

@@ -1,0 +1,660 @@
+// sweep2d_ring.cuh -- the X-Y transport sweep (K1) of the angular-moment source modes
+// (isotropic, linear kernel) with one grid row per wavefront step and the cell rows
+// staged through per-lane rings in shared memory.
+//
+// Same cell equations, work items (up to G ordinates of one quadrant of one sample) and
+// moment accumulators as the other X-Y sweeps.  Lanes are numbered from the inflow face;
+// lane p owns the 4 cells at distance 4p .. 4p+3 from it in every row, and lane d of a
+// warp sweeps row t - d at the warp's step t, so the x-edge flux passes one lane per step
+// by a shuffle and the y-edge fluxes stay in registers.  Warp w of a wide row runs
+// kLag * 8 steps behind warp w - 1 and takes the x-edges from a shared-memory ring; the
+// warps meet at one CTA barrier per 8 steps.
+//
+// Memory.  The lanes of a warp sit on 32 different rows, so a direct access of the warp
+// would touch 32 cache lines for 512 bytes, and the L1 would be the limit (one line per
+// cycle: 32 cycles per access, three accesses per step, against ~100 cycles of
+// arithmetic).  Instead each 8-lane group copies 128 contiguous bytes of one row per step
+// (cp.async, row t + kAhead - 8 * group), every lane into its own column of a 16-row ring,
+// and reads its own cells when its step comes; it leaves the moments in the same slot,
+// and the group adds them to the accumulator row by row, 128 contiguous bytes at a time
+// (red.global.add.v4), once its last lane has passed.  A lane only ever touches its own
+// column of the ring, so no barrier is involved.
+//
+// Arithmetic.  With f = 2 (diamond difference) or 1 (step), a = f|c|/dx, b = f|s|/dy,
+// d = sigma_T + a + b, the edge fluxes are kept scaled so that the source enters every
+// ordinate of a pack with coefficient one:
+//   uniform sigma_T: X = x d / f, P = b y:    t = S + P, X' = alpha X + t,
+//     DD:   alpha = (a - b - sigma_T) / d, sum = X + X', P' = 2 b / d sum - P,
+//     step: alpha = a / d,                 sum = X',     P' = b / d sum,
+//     moment += (w / d) sum;
+//   varying sigma_T: X = a x, P = b y: psi = (S + X + P) / d, X' = f a psi - X (DD) or
+//     a psi, P' likewise, moment += w psi.
+// The uniform case takes five packed FP32x2 operations per cell and ordinate pair and its
+// upwind chain is one FMA per cell.  The packed instructions take no negated operand, so
+// the DD closure keeps -P at odd steps (and the varying case -X at odd cells): P' = c - P
+// becomes (-P') = P - c, one FMA with a negated constant either way.
+#pragma once
+#include <type_traits>
+
+#include "rom_internal.cuh"
+
+namespace romk {
+namespace {
+
+constexpr int kRows = 16;    // rows of a ring
+constexpr int kAhead = 7;    // rows a group copies ahead of its first lane's step: the slot
+                             // of row r - 16 is drained one step before row r is copied
+constexpr int kGrp = 8;      // steps between CTA barriers; lanes of a 128-byte group
+constexpr int kLag = 5;      // groups of steps a warp runs behind its upstream warp: row r
+                             // leaves that warp 9 steps before it is needed, and is read
+                             // one step early, so a barrier lies between
+constexpr int kEdgeRows = 32;
+
+template <int G>
+struct RingPack {
+    static constexpr int N = G / 2;
+};
+__device__ __forceinline__ float2 qfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 qmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 qadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 qsplat(float s) { return make_float2(s, s); }
+__device__ __forceinline__ float2 qneg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float qrcp(float a)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));  // within 1 ulp; a >= sigma_T > 0
+    return r;
+}
+__device__ __forceinline__ void qset(float2 &a, int i, float v)
+{
+    if (i) a.y = v;
+    else a.x = v;
+}
+__device__ __forceinline__ float qget(const float2 &a, int i) { return i ? a.y : a.x; }
+__device__ __forceinline__ float f4(const float4 &v, int r)
+{
+    return r == 0 ? v.x : r == 1 ? v.y : r == 2 ? v.z : v.w;
+}
+__device__ __forceinline__ unsigned ring_u32(const void *p)
+{
+    return (unsigned)__cvta_generic_to_shared(p);
+}
+// Shared- and global-memory accesses of a step, all kept in program order.  The predicated
+// ones skip by a predicate, not a branch, which would split the step's instructions: a copy
+// or reduction whose row is outside [0, lim) (lim = 0: a chunk without cells), a store of a
+// lane without cells.
+__device__ __forceinline__ float4 lds4(unsigned p)
+{
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(p));
+    return v;
+}
+__device__ __forceinline__ void sts4(unsigned p, const float4 &v)
+{
+    asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(p), "f"(v.x), "f"(v.y), "f"(v.z),
+                 "f"(v.w)
+                 : "memory");
+}
+template <int C>
+__device__ __forceinline__ void sts_cells(const unsigned *p, unsigned off, const float *v, bool on)
+{
+    if constexpr (C == 8)
+        asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %10, 0;\n\t"
+                     "@q st.shared.v4.f32 [%0], {%2,%3,%4,%5};\n\t"
+                     "@q st.shared.v4.f32 [%1], {%6,%7,%8,%9};\n\t}" ::"r"(p[0] + off),
+                     "r"(p[1] + off), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]),
+                     "f"(v[5]), "f"(v[6]), "f"(v[7]), "r"((unsigned)on)
+                     : "memory");
+    else
+        asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %5, 0;\n\t"
+                     "@q st.shared.v4.f32 [%0], {%1,%2,%3,%4};\n\t}" ::"r"(p[0] + off), "f"(v[0]),
+                     "f"(v[1]), "f"(v[2]), "f"(v[3]), "r"((unsigned)on)
+                     : "memory");
+}
+template <int OFF>  // bytes from src to the chunk
+__device__ __forceinline__ void ring_copy(unsigned dst, const float *src, int row, int lim)
+{
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.lt.u32 q, %2, %3;\n\t"
+                 "@q cp.async.cg.shared.global [%0], [%1+%4], 16;\n\t}" ::"r"(dst), "l"(src),
+                 "r"(row), "r"(lim), "n"(OFF)
+                 : "memory");
+}
+template <int OFF>
+__device__ __forceinline__ void ring_red(float *p, const float4 &v, int row, int lim)
+{
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.lt.u32 q, %5, %6;\n\t"
+                 "@q red.global.add.v4.f32 [%0+%7], {%1,%2,%3,%4};\n\t}" ::"l"(p), "f"(v.x),
+                 "f"(v.y), "f"(v.z), "f"(v.w), "r"(row), "r"(lim), "n"(OFF)
+                 : "memory");
+}
+// test hook: a wait, bounded in time, on an mbarrier that nothing completes
+__device__ __forceinline__ bool ring_never_wait(unsigned long long *b, unsigned long long budget_ns)
+{
+    unsigned long long t0;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+    for (;;) {
+        unsigned ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(ring_u32(b)), "r"(0u)
+            : "memory");
+        if (__all_sync(0xffffffffu, ok != 0)) return true;
+        unsigned long long t;
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+        if (__any_sync(0xffffffffu, t - t0 > budget_ns)) return false;
+    }
+}
+
+// arrays staged per warp: the source moments (their slots take the flux moments), sigma_T
+__host__ __device__ constexpr int ring_arrays(int mom, bool homog) { return mom + (homog ? 0 : 1); }
+// shared memory of a CTA: the warps' rings, their incoming x-edges, 16 zero bytes
+__host__ __device__ constexpr int ring_bytes(int mom, bool homog, int nwarps, int G, int C)
+{
+    return nwarps * (ring_arrays(mom, homog) * kRows * 32 * C + kEdgeRows * G) * 4 + 16;
+}
+
+template <int C, int G, int MOM, int SCHEME, bool HOMOG, bool XNEG, bool RAGGED, bool EDGE>
+__device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd,
+                                          const SweepItem &it, char *smem)
+{
+    constexpr int N = RingPack<G>::N;
+    constexpr int NA = ring_arrays(MOM, HOMOG);
+    constexpr unsigned kRowB = 32 * C * 4, kArrB = kRows * kRowB;  // bytes of a ring row, a ring
+    constexpr int CH = C / 4;  // 16-byte chunks of a lane's cells
+    constexpr unsigned kMask = kArrB - 1;
+    constexpr unsigned kEdgeB = kEdgeRows * G * 4;
+    constexpr bool DD = SCHEME == 0;
+    const int nw = blockDim.x >> 5, lane = threadIdx.x & 31;
+    const int w = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);  // (uniform)
+    const int L = (gd.I + C - 1) / C;  // lanes that own cells
+    const int p = 32 * w + lane;
+    const bool on = p < L;
+    const int col = on ? C * (XNEG ? L - 1 - p : p) : 0;
+    const bool yneg = (it.quad >> 1) & 1;
+    const int J = gd.J;
+    const float fdd = DD ? 2.f : 1.f;
+
+    // per-ordinate constants (see the head of the file); an empty slot has weight zero
+    float2 k1[N], k2[N], k2n[N], km[N], kmc[N], kms[N], kc[N], ks[N], ab[N], lx[N], wl[N];
+    int ord[G];
+    float inj_x[G], inj_y[G];  // boundary value -> scaled edge flux
+#pragma unroll
+    for (int k = 0; k < G; ++k) {
+        float c = 0.f, s = 0.f, wt = 0.f;
+        ord[k] = it.ord[0];
+        if (k < it.n) {
+            ord[k] = it.ord[k];
+            c = A.oc[ord[k]];
+            s = A.os[ord[k]];
+            wt = A.ow[ord[k]];
+        }
+        const int pk = k >> 1, i = k & 1;
+        const float a = fdd * fabsf(c) * gd.inv_dx, b = fdd * fabsf(s) * gd.inv_dy;
+        const float st = A.sigma_t_homog;
+        const float rd = HOMOG ? 1.f / (st + a + b) : 1.f;
+        const float wm = HOMOG ? wt * rd : wt;
+        qset(k1[pk], i, HOMOG ? (DD ? (a - b - st) * rd : a * rd) : fdd * a);
+        qset(k2[pk], i, HOMOG ? fdd * b * rd : fdd * b);
+        qset(ab[pk], i, a + b);
+        qset(km[pk], i, wm);
+        qset(kmc[pk], i, wm * c);
+        qset(kms[pk], i, wm * s);
+        qset(kc[pk], i, c);
+        qset(ks[pk], i, s);
+        // leakage: w |s| dx y = (w dx dy / f) P; w |c| dy x = w |c| dy f rd X, or (w dx dy / f) X
+        qset(wl[pk], i, wt * gd.dx * gd.dy / fdd);
+        const float lo = HOMOG ? wt * fabsf(c) * gd.dy * fdd * rd : wt * gd.dx * gd.dy / fdd;
+        qset(lx[pk], i, (A.leak != nullptr && p == L - 1) ? lo : 0.f);
+        inj_x[k] = HOMOG ? (st + a + b) / fdd : a;
+        inj_y[k] = b;
+    }
+#pragma unroll
+    for (int q = 0; q < N; ++q) k2n[q] = qneg(k2[q]);
+    // lane 0 takes no x-edge from the shuffle
+    const float2 neg1 = qsplat(-1.f), k0 = qsplat(lane == 0 ? 0.f : 1.f);
+    float2 k1f[N];
+#pragma unroll
+    for (int q = 0; q < N; ++q) k1f[q] = qmul(k1[q], k0);
+    // real[rr]: the cell at sweep position rr (column XNEG ? 3 - rr : rr) is inside the grid
+    bool real[C];
+#pragma unroll
+    for (int rr = 0; rr < C; ++rr)
+        real[rr] = !RAGGED || col + (XNEG ? C - 1 - rr : rr) < gd.I;
+
+    // The lane's rings, all zero at first (sigma_T one): rows before the grid's first sweep
+    // zeros, and so does a lane without cells.  Slots go by step: the cells of step t are in
+    // slot t mod 16 of every lane; the row copied at step t is the one of the lane's step
+    // t + kAhead + (lane & 7), and the row drained, 15 rows before it, sits in the next slot.
+    // Of 8 cells a lane's two halves trade places on every other 4 lanes (bank conflicts).
+    // The lane copies and drains CH chunks of its group's row: lane e those of the group's
+    // lanes e (C = 4), or e / 2 and 4 + e / 2 (C = 8), which keeps every access of the group
+    // to 128 contiguous bytes.
+    const unsigned rings = ring_u32(smem) + w * NA * kArrB;
+    const int sw = CH == 2 ? (lane >> 2) & 1 : 0;
+    unsigned own[CH];
+#pragma unroll
+    for (int h = 0; h < CH; ++h) own[h] = rings + lane * C * 4 + ((h ^ sw) * 16);
+    for (int m = 0; m < NA; ++m)
+        for (int r = 0; r < kRows; ++r) {
+            const float z = m == MOM ? 1.f : 0.f;
+#pragma unroll
+            for (int h = 0; h < CH; ++h) sts4(own[h] + m * kArrB + r * kRowB, make_float4(z, z, z, z));
+        }
+    __syncwarp();
+    const unsigned edges = ring_u32(smem) + nw * NA * kArrB;
+    if constexpr (EDGE) {
+        for (int k = threadIdx.x; k < nw * kEdgeRows * G + 4; k += blockDim.x)
+            ((float *)(smem + (size_t)nw * NA * kArrB))[k] = 0.f;
+        __syncthreads();
+    }
+    // lane 0 reads the x-edges of its warp, the others the zeros after the last ring
+    const unsigned edge_in = lane == 0 ? edges + w * kEdgeB : edges + nw * kEdgeB;
+    const unsigned edge_sel = lane == 0 ? kEdgeB - 1 : 0;
+    const unsigned edge_out = edges + (w + 1) * kEdgeB;
+
+    const long long so = A.soff ? A.soff[it.sample] : (long long)it.sample * MOM * gd.cells;
+    const long long rs = yneg ? -(long long)gd.NXP : (long long)gd.NXP;
+    const long long cells = gd.cells;
+    const int grp8 = lane & ~7;  // 8 * the lane's group
+
+    float2 P[C][N], X[N];
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+        X[q] = qsplat(0.f);
+#pragma unroll
+        for (int r = 0; r < C; ++r) P[r][q] = qsplat(0.f);
+    }
+    double leak = 0.0;
+    // With an inflow the incoming y-edges wait in P, held by zero constants (k2, and the
+    // x leakage's lx), until the lane's first row: the rows before it compute numbers that
+    // reach no cell of the grid.  The step of that row finds P negated if it is odd.
+    bool held = false;
+    float2 k2s[N], lxs[N];  // (EDGE)
+    if constexpr (EDGE) {
+        held = A.inflow != nullptr;
+        if (held) {
+#pragma unroll
+            for (int r = 0; r < C; ++r)
+#pragma unroll
+                for (int k = 0; k < G; ++k)
+                    if (on && col + r < gd.I && k < it.n) {
+                        const float b = inj_y[k] * A.inflow[(long long)ord[k] * A.inflow_stride +
+                                                            2 * J + (yneg ? gd.I : 0) + col + r];
+                        qset(P[r][k >> 1], k & 1, DD && (lane & 1) ? -b : b);
+                        leak -= (double)(qget(wl[k >> 1], k & 1) * b);
+                    }
+        }
+#pragma unroll
+        for (int q = 0; q < N; ++q) {
+            k2s[q] = k2[q];
+            lxs[q] = lx[q];
+            if (held) k2[q] = k2n[q] = lx[q] = qsplat(0.f);
+        }
+    }
+    float lk_s = 0.f, lk_c = 0.f;  // compensated (Kahan) sum of the groups' x-edge terms
+    float2 lk[N];
+#pragma unroll
+    for (int q = 0; q < N; ++q) lk[q] = qsplat(0.f);
+
+    // Groups of 8 steps of the warp: steps -8 .. J + 7 + 8 * (its last lanes' group); a warp
+    // starts kLag groups after the one upstream.  nwl: warps that own cells (a batch's
+    // narrower grid leaves some without).
+    const int nwl = (L + 31) / 32;
+    auto groups = [&](int lanes) { return 1 + (J + 8 + ((lanes - 1) & ~7) + kGrp - 1) / kGrp; };
+    const int n_grp_l = groups(L - 32 * (nwl - 1)), n_grp_f = groups(32);
+    const int n_grp_w = w >= nwl ? 0 : w == nwl - 1 ? n_grp_l : n_grp_f;
+    const int n_grp = nwl == 1 ? n_grp_l
+                               : max(n_grp_f + kLag * (nwl - 2), n_grp_l + kLag * (nwl - 1));
+    const bool feeds = lane == 31 && w < nwl - 1;
+
+    bool past = false;
+    int t = -kGrp;
+    const long long o0 = so + (yneg ? (long long)(J - 1) * gd.NXP : 0);
+    int frow = t + kAhead - grp8;  // the row copied at step t
+    int lim[CH];              // J, or 0 for a chunk without cells
+    unsigned fd[CH];          // the slot copied into (the row drained is in the next one)
+    const int dl0 = CH == 1 ? lane & 7 : (lane & 7) >> 1, half = CH == 1 ? 0 : lane & 1;
+#pragma unroll
+    for (int h = 0; h < CH; ++h) {
+        const int dl = dl0 + 4 * h;  // the group's lane whose cells they are
+        lim[h] = 32 * w + grp8 + dl < L ? J : 0;
+        fd[h] = (unsigned)(t + kAhead + dl) % kRows * kRowB;
+    }
+    const unsigned place = rings + (grp8 + dl0) * C * 4 + half * 16;  // of the first chunk
+    constexpr unsigned kPlace1 = 4 * C * 4;  // the second: 4 lanes on, halves exchanged
+    const unsigned place1 = CH == 2 ? (place ^ 16) + kPlace1 : 0;
+    constexpr int kChunk1 = (XNEG ? -1 : 1) * 4 * C * 4;  // bytes between the chunks' cells
+    const int cd = C * (XNEG ? L - 1 - (32 * w + grp8 + dl0) : 32 * w + grp8 + dl0) + 4 * half;
+    const float *src = A.src + o0 + cd + frow * rs;
+    const float *sig = HOMOG ? nullptr : A.sigma_t + gd.off + (o0 - so) + cd + frow * rs;
+    float *acc = A.part + o0 + cd + (frow - kRows + 1) * rs;
+    unsigned cs = 0;             // slot of the step's cells (step 0: slot 0)
+    unsigned eo = 0;             // offset of the x-edges of row t + 1 (and of row t - 31)
+
+    float4 S[NA][CH];                            // the cells of the next step
+    float4 E = make_float4(0.f, 0.f, 0.f, 0.f);  // its incoming x-edge (lane 0)
+
+    auto fill = [&]() {
+#pragma unroll
+        for (int m = 0; m < NA; ++m) {
+            const float *p = m < MOM ? src + m * cells : sig;
+            ring_copy<0>(place + m * kArrB + fd[0], p, frow, lim[0]);
+            if constexpr (CH == 2)
+                ring_copy<kChunk1>(place1 + m * kArrB + fd[CH - 1], p, frow, lim[CH - 1]);
+        }
+        src += rs;
+        if constexpr (!HOMOG) sig += rs;
+        ++frow;
+#pragma unroll
+        for (int h = 0; h < CH; ++h) fd[h] = (fd[h] + kRowB) & kMask;
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        // this step's copies and those of the five before it may still be in flight: a row
+        // is read 6 copies after its own
+        asm volatile("cp.async.wait_group 6;" ::: "memory");
+        if constexpr (CH == 2) __syncwarp();  // (C = 4: a lane copies and drains its own cells)
+    };
+    auto load = [&]() {
+#pragma unroll
+        for (int m = 0; m < NA; ++m)
+#pragma unroll
+            for (int h = 0; h < CH; ++h) S[m][h] = lds4(own[h] + m * kArrB + cs);
+        if constexpr (EDGE) {
+            const unsigned ep = edge_in + (eo & edge_sel);
+            if constexpr (N == 2) E = lds4(ep);
+            else
+                asm volatile("ld.shared.v2.f32 {%0,%1}, [%2];" : "=f"(E.x), "=f"(E.y) : "r"(ep));
+        }
+    };
+
+    // One step.  EV: some lane passes its first or last row in this group of steps; ODD: P
+    // holds its negative.
+    auto step = [&](auto events, auto odd) {
+        constexpr bool EV = decltype(events)::value;
+        constexpr bool ODD = DD && decltype(odd)::value;
+        fill();
+        // the moments of the row that the group's last lane finished at the step before
+        // (fill has moved on to its slot)
+        float4 D[MOM][CH];
+#pragma unroll
+        for (int m = 0; m < MOM; ++m)
+#pragma unroll
+            for (int h = 0; h < CH; ++h)
+                D[m][h] = lds4((h ? place1 : place) + m * kArrB + fd[h]);
+        const unsigned slot = cs;
+        float4 V[NA][CH];
+#pragma unroll
+        for (int m = 0; m < NA; ++m)
+#pragma unroll
+            for (int h = 0; h < CH; ++h) V[m][h] = S[m][h];
+        float2 x[C + 1][N], sm[C][N];
+#pragma unroll
+        for (int q = 0; q < N; ++q) {
+            const float2 e = q == 0 ? make_float2(E.x, E.y) : make_float2(E.z, E.w);
+            x[0][q] = EDGE ? qfma(X[q], k0, e) : X[q];
+        }
+        cs = (cs + kRowB) & kMask;
+        if constexpr (EDGE) eo = (eo + G * 4) & (kEdgeB - 1);
+        load();
+        if constexpr (EV) {
+            const int row = t - lane;
+            if (EDGE && held && row == 0) {  // the lane's first row: its y-edges come free
+                held = false;
+#pragma unroll
+                for (int q = 0; q < N; ++q) {
+                    k2[q] = k2s[q];
+                    k2n[q] = qneg(k2s[q]);
+                    lx[q] = lxs[q];
+                }
+            }
+            if (row == J) {  // past the last row the y-edges stay and nothing counts
+                past = true;
+#pragma unroll
+                for (int q = 0; q < N; ++q) k2[q] = k2n[q] = lx[q] = qsplat(0.f);
+            }
+        }
+#pragma unroll
+        for (int rr = 0; rr < C; ++rr) {
+            const int r = XNEG ? C - 1 - rr : rr;
+#pragma unroll
+            for (int q = 0; q < N; ++q) {
+                float2 tt;
+                if constexpr (MOM == 3) {
+                    const float2 s =
+                        qfma(kc[q], qsplat(f4(V[MOM == 3 ? 1 : 0][r / 4], r % 4)),
+                             qfma(ks[q], qsplat(f4(V[MOM == 3 ? 2 : 0][r / 4], r % 4)), qsplat(f4(V[0][r / 4], r % 4))));
+                    tt = ODD ? qfma(P[r][q], neg1, s) : qadd(s, P[r][q]);
+                } else {
+                    const float s = f4(V[0][r / 4], r % 4);
+                    tt = ODD ? make_float2(s - P[r][q].x, s - P[r][q].y)
+                             : make_float2(s + P[r][q].x, s + P[r][q].y);
+                }
+                const bool first = !EDGE && rr == 0;  // lane 0 takes no x-edge
+                if constexpr (HOMOG) {
+                    float2 xn = qfma(first ? k1f[q] : k1[q], x[rr][q], tt);
+                    if (RAGGED && !real[rr]) xn = first ? qmul(x[rr][q], k0) : x[rr][q];
+                    x[rr + 1][q] = xn;
+                    sm[rr][q] = !DD ? xn : first ? qfma(x[rr][q], k0, xn) : qadd(x[rr][q], xn);
+                } else {
+                    if (first) x[0][q] = qmul(x[0][q], k0);
+                    const float s = f4(V[NA - 1][r / 4], r % 4);
+                    const float2 rd = make_float2(qrcp(s + ab[q].x), qrcp(s + ab[q].y));
+                    // DD: x[] holds the negative at odd cells
+                    const float2 num =
+                        (DD && (rr & 1)) ? qfma(x[rr][q], neg1, tt) : qadd(tt, x[rr][q]);
+                    const float2 psi = qmul(num, rd);
+                    sm[rr][q] = psi;
+                    float2 xn = DD ? qfma((rr & 1) ? k1[q] : qneg(k1[q]), psi, x[rr][q])
+                                   : qmul(k1[q], psi);
+                    if (RAGGED && !real[rr]) xn = DD ? qneg(x[rr][q]) : x[rr][q];
+                    x[rr + 1][q] = xn;
+                }
+            }
+        }
+        // the x-edges to the next lane, and from the last lane to the next warp
+#pragma unroll
+        for (int q = 0; q < N; ++q) {
+            X[q].x = __shfl_up_sync(0xffffffffu, x[C][q].x, 1);
+            X[q].y = __shfl_up_sync(0xffffffffu, x[C][q].y, 1);
+        }
+        if constexpr (EDGE) {
+            if constexpr (N == 2)
+                asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %5, 0;\n\t"
+                             "@q st.shared.v4.f32 [%0], {%1,%2,%3,%4};\n\t}" ::"r"(edge_out + eo),
+                             "f"(x[C][0].x), "f"(x[C][0].y), "f"(x[C][N - 1].x),
+                             "f"(x[C][N - 1].y), "r"((unsigned)feeds)
+                             : "memory");
+            else
+                asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %3, 0;\n\t"
+                             "@q st.shared.v2.f32 [%0], {%1,%2};\n\t}" ::"r"(edge_out + eo),
+                             "f"(x[C][0].x), "f"(x[C][0].y), "r"((unsigned)feeds)
+                             : "memory");
+        }
+        float v[MOM][C];
+#pragma unroll
+        for (int rr = 0; rr < C; ++rr) {
+            const int r = XNEG ? C - 1 - rr : rr;
+            float2 m[MOM];
+#pragma unroll
+            for (int q = 0; q < N; ++q) {
+                const float2 s = sm[rr][q];
+                if (!RAGGED || real[rr])
+                    P[r][q] = DD ? qfma(ODD ? k2[q] : k2n[q], s, P[r][q])
+                                 : EV && (held || past) ? P[r][q] : qmul(k2[q], s);
+#pragma unroll
+                for (int k = 0; k < MOM; ++k) {
+                    const float2 kw = k == 0 ? km[q] : k == 1 ? kmc[q] : kms[q];
+                    m[k] = q == 0 ? qmul(kw, s) : qfma(kw, s, m[k]);
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < MOM; ++k) v[k][r] = (!RAGGED || real[rr]) ? m[k].x + m[k].y : 0.f;
+        }
+#pragma unroll
+        for (int k = 0; k < MOM; ++k) sts_cells<C>(own, k * kArrB + slot, v[k], on);
+#pragma unroll
+        for (int q = 0; q < N; ++q) lk[q] = qfma(lx[q], x[C][q], lk[q]);
+#pragma unroll
+        for (int m = 0; m < MOM; ++m) {
+            ring_red<0>(acc + m * cells, D[m][0], frow - kRows, lim[0]);
+            if constexpr (CH == 2)
+                ring_red<kChunk1>(acc + m * cells, D[m][CH - 1], frow - kRows, lim[CH - 1]);
+        }
+        acc += rs;
+        ++t;
+    };
+
+    // x inflow, scaled, of rows r0 .. r0 + 7: lane e takes ordinate e % G of row r0 + e / G
+    constexpr int kPre = (kGrp * G + 31) / 32;
+    float pre[kPre];
+    auto fetch = [&](int r0) {
+#pragma unroll
+        for (int e = 0; e < kPre; ++e) {
+            const int k = (32 * e + lane) % G, rr = r0 + (32 * e + lane) / G;
+            float ix = 0.f, lw = 0.f;
+            int o = 0;
+#pragma unroll
+            for (int kk = 0; kk < G; ++kk)
+                if (kk == k && kk < it.n) {
+                    ix = inj_x[kk];
+                    lw = A.ow[ord[kk]] * fabsf(A.oc[ord[kk]]) * gd.dy;
+                    o = ord[kk];
+                }
+            float b = 0.f;
+            if (32 * e + lane < kGrp * G && rr >= 0 && rr < J)
+                b = A.inflow[(long long)o * A.inflow_stride + (XNEG ? J : 0) +
+                             (yneg ? J - 1 - rr : rr)];
+            pre[e] = ix * b;
+            leak -= (double)(lw * b);
+        }
+    };
+    if (EDGE && w == 0 && A.inflow != nullptr) fetch(1 - kGrp);
+    for (int g = 0; g < n_grp; ++g) {
+        const int gl = g - kLag * w;  // the warp's own group of steps
+        if (gl >= 0 && gl < n_grp_w) {
+            if (EDGE && w == 0 && A.inflow != nullptr) {
+                // x inflow of the rows this group reads (t + 1 .. t + 8), loaded a group ago
+#pragma unroll
+                for (int e = 0; e < kPre; ++e)
+                    if (32 * e + lane < kGrp * G)
+                        ((float *)(smem + (size_t)nw * NA * kArrB))
+                            [(unsigned)(t + 1 + (32 * e + lane) / G) % kEdgeRows * G +
+                             (32 * e + lane) % G] = pre[e];
+                __syncwarp();
+                fetch(t + 1 + kGrp);
+            }
+            if (gl == 0) {  // the first rows on their way
+#pragma unroll 1
+                for (int u = 0; u < kGrp; ++u) fill();
+                acc += kGrp * rs;
+                t = 0;
+                load();
+            } else if (t + kGrp > J || (EDGE && t < 32 && A.inflow != nullptr)) {
+#pragma unroll 1
+                for (int u = 0; u < kGrp; u += 2) {
+                    step(std::true_type{}, std::false_type{});
+                    step(std::true_type{}, std::true_type{});
+                }
+            } else {
+#pragma unroll 1
+                for (int u = 0; u < kGrp; u += 2) {
+                    step(std::false_type{}, std::false_type{});
+                    step(std::false_type{}, std::true_type{});
+                }
+            }
+            const float yv = (N == 2 ? (lk[0].x + lk[0].y) + (lk[N - 1].x + lk[N - 1].y)
+                                     : lk[0].x + lk[0].y) - lk_c;
+            const float tt = lk_s + yv;
+            lk_c = (tt - lk_s) - yv;
+            lk_s = tt;
+#pragma unroll
+            for (int q = 0; q < N; ++q) lk[q] = qsplat(0.f);
+        }
+        if (EDGE && nw > 1) __syncthreads();
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (A.leak != nullptr) {  // the outgoing y-edges; one FP64 add per warp
+        float lo = 0.f;
+#pragma unroll
+        for (int r = 0; r < C; ++r)
+            if (on && col + r < gd.I)
+#pragma unroll
+                for (int q = 0; q < N; ++q) lo += wl[q].x * P[r][q].x + wl[q].y * P[r][q].y;
+        // (the last row's step J - 1 + lane left -P if it was even)
+        leak += (double)(DD && ((J - 1 + lane) & 1) == 0 ? -lo : lo) + ((double)lk_s - (double)lk_c);
+#pragma unroll
+        for (int dd = 16; dd > 0; dd >>= 1) leak += __shfl_xor_sync(0xffffffffu, leak, dd);
+        if (lane == 0 && leak != 0.0) atomicAdd(A.leak + it.sample, leak);
+    }
+}
+
+template <int C, int G, int MOM, int SCHEME, bool HOMOG, bool EDGE, int MAXT>
+__global__ void __launch_bounds__(MAXT) sweep2d_ring_kernel(const SweepArgs A)
+{
+    extern __shared__ __align__(1024) char ring_smem[];
+    const SweepItem it = A.items[blockIdx.x];
+    if (!A.active[it.sample]) return;
+    // Several grids vary in sigma_T: those kernels take every grid from the table, one grid
+    // too (a choice here between the table and the arguments' fields was miscompiled: the
+    // width alone stayed the arguments').
+    GridDesc gd{A.I, A.J, A.NXP, A.inv_dx, A.inv_dy, A.dx, A.dy, 0, A.cells};
+    if constexpr (!HOMOG) gd = A.gdesc[it.grid];
+    if (A.stall) {  // test hook: every warp waits on a barrier that nothing completes
+        __shared__ unsigned long long never;
+        if (threadIdx.x == 0)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(ring_u32(&never))
+                         : "memory");
+        __syncthreads();
+        if (!ring_never_wait(&never, A.wait_ns)) {
+            if ((threadIdx.x & 31) == 0) atomicOr(A.err, 1);
+            return;
+        }
+    }
+    const bool ragged = gd.I % C != 0;
+    if (it.quad & 1) {
+        if (ragged) ring_item<C, G, MOM, SCHEME, HOMOG, true, true, EDGE>(A, gd, it, ring_smem);
+        else ring_item<C, G, MOM, SCHEME, HOMOG, true, false, EDGE>(A, gd, it, ring_smem);
+    } else {
+        if (ragged) ring_item<C, G, MOM, SCHEME, HOMOG, false, true, EDGE>(A, gd, it, ring_smem);
+        else ring_item<C, G, MOM, SCHEME, HOMOG, false, false, EDGE>(A, gd, it, ring_smem);
+    }
+}
+
+template <int C, int G, int MOM, int SCHEME, bool HOMOG, bool EDGE>
+cudaError_t ring_launch_k(const SweepArgs &a, int n_items, int nwarps, cudaStream_t st)
+{
+    const int bytes = ring_bytes(MOM, HOMOG, nwarps, G, C);
+    auto k = sweep2d_ring_kernel<C, G, MOM, SCHEME, HOMOG, EDGE, EDGE ? 256 : 64>;
+    if (bytes > 48 * 1024) {
+        const cudaError_t e =
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e != cudaSuccess) return e;
+    }
+    k<<<n_items, 32 * nwarps, bytes, st>>>(a);
+    return cudaGetLastError();
+}
+
+template <int MOM, int SCHEME, bool HOMOG>
+cudaError_t ring_launch(const SweepArgs &a, int n_items, int C, int G, cudaStream_t st)
+{
+    const int nw = (a.I + 32 * C - 1) / (32 * C);
+    const bool inflow = a.inflow != nullptr;
+    // items of one ordinate run on the two-ordinate kernel (the empty slot has weight zero)
+#define RING_K(CC, GG)                                                                            \
+    return nw > 1 || inflow ? ring_launch_k<CC, GG, MOM, SCHEME, HOMOG, true>(a, n_items, nw, st) \
+                            : ring_launch_k<CC, GG, MOM, SCHEME, HOMOG, false>(a, n_items, nw, st)
+    if (C == 8) {
+        if (G == 4) RING_K(8, 4);
+        RING_K(8, 2);
+    }
+    if (G == 4) RING_K(4, 4);
+    RING_K(4, 2);
+#undef RING_K
+}
+
+}  // namespace
+}  // namespace romk

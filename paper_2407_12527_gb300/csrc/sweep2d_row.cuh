@@ -556,25 +556,23 @@ cudaError_t row_launch(const SweepArgs &a, int n_items, int nwarps, int G, bool 
     const dim3 grid(n_items), block(32 * nwarps);
     const bool multi = nwarps > 1, inflow = a.inflow != nullptr;
 #define ROW_K(GG, HH, MM, II) sweep2d_row_kernel<GG, MOM, SCHEME, HH, BATCH, MM, II><<<grid, block, 0, st>>>(a)
+// (moment modes: rows that fit one warp run on sweep2d_ring.cuh)
+#define ROW_M(GG, HH, II)                                    \
+    do {                                                     \
+        if constexpr (MOM == 0) {                            \
+            if (multi) ROW_K(GG, HH, true, II);              \
+            else ROW_K(GG, HH, false, II);                   \
+        } else ROW_K(GG, HH, true, II);                      \
+    } while (0)
 #define ROW_G(GG, HH)                                        \
     do {                                                     \
-        if (multi) {                                         \
-            if (inflow) ROW_K(GG, HH, true, true);           \
-            else ROW_K(GG, HH, true, false);                 \
-        } else {                                             \
-            if (inflow) ROW_K(GG, HH, false, true);          \
-            else ROW_K(GG, HH, false, false);                \
-        }                                                    \
+        if (inflow) ROW_M(GG, HH, true);                     \
+        else ROW_M(GG, HH, false);                           \
     } while (0)
     if constexpr (BATCH) {
         (void)homog;  // several grids: sigma_T read per cell, vacuum boundaries
-        if (G == 4) {
-            if (multi) ROW_K(4, false, true, false);
-            else ROW_K(4, false, false, false);
-        } else {
-            if (multi) ROW_K(2, false, true, false);
-            else ROW_K(2, false, false, false);
-        }
+        if (G == 4) ROW_K(4, false, true, false);
+        else ROW_K(2, false, true, false);
     } else {
         if (G == 4) {
             if (homog) ROW_G(4, true);
@@ -585,6 +583,7 @@ cudaError_t row_launch(const SweepArgs &a, int n_items, int nwarps, int G, bool 
         }
     }
 #undef ROW_G
+#undef ROW_M
 #undef ROW_K
     return cudaGetLastError();
 }
