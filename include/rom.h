@@ -89,10 +89,11 @@ typedef struct rom_options {
                      /* > 0: the host reads the number of unconverged samples after every  */
                      /* check_every sweeps                                                 */
     int tile_g;      /* ordinates per sweep work item: 1, 2 or 4; 0 = chosen from the      */
-                     /* problem size (and rows_per_step with it); -1 = measured: at the     */
-                     /* first solve of a problem layout the candidate shapes (with the     */
-                     /* one-row moment sweep: its sizes) are timed on a few sweeps and the fastest is kept   */
-                     /* (until the grid, the ordinate layout or the kernel changes)        */
+                     /* problem size (and rows_per_step with it); -1 = measured: at the    */
+                     /* first solve of a problem layout the candidate shapes (of the       */
+                     /* one-row sweep, where it runs) are timed on a few sweeps and the    */
+                     /* fastest is kept (until the grid, the ordinate layout or the kernel */
+                     /* changes)                                                           */
     int time_kernels;/* 0; 1 records CUDA events around every sweep launch (host-driven     */
                      /* loop, check_every >= 1 is then used, 1 if it is 0) and reports the  */
                      /* summed sweep-kernel time in rom_stats.sweep_ms                     */
@@ -106,10 +107,11 @@ typedef struct rom_options {
                      /* 128 ordinates per sample and 2048 samples per context, else        */
                      /* ROM_ERR_UNSUPPORTED)                                               */
     int rows_per_step; /* X-Y sweep: grid rows a lane advances per wavefront step; 0 =     */
-                     /* chosen: with tile_g = 0 in the isotropic and linear-kernel moment  */
-                     /* modes 1, with tile_g = -1 the measured choice (1, 2 or 4), else 4;  */
-                     /* 1, 2 or 4 forces it (2 only in the moment modes: the dense operator */
-                     /* mode runs 4 then); other values are ROM_ERR_INVALID_ARG            */
+                     /* chosen: with tile_g = 0 the library's choice (1, or 4 on very wide */
+                     /* grids), with tile_g = -1 the measured one (1, 2 or 4), else 4; 1, 2 */
+                     /* or 4 forces it (2 only in the isotropic and linear-kernel moment   */
+                     /* modes: the dense operator mode runs 4 then); other values are      */
+                     /* ROM_ERR_INVALID_ARG                                                */
     int diverge_window; /* 16: a sample whose change ||phi^k - phi^{k-1}||_2 grew in this  */
                      /* many consecutive sweeps (while above tol) stops as diverged         */
                      /* (ROM_ERR_DIVERGED); 0 turns the test off                            */

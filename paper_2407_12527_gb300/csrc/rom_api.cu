@@ -379,9 +379,10 @@ bool ring_sweep(const rom_ctx *ctx)
 int choose_rows(const rom_ctx *ctx)
 {
     if (ctx->dim != 2) return 4;
-    if (source_mode(ctx) == 0) {  // dense operator mode: the 4-row or the one-row kernel
+    if (source_mode(ctx) == 0) {  // dense operator mode: the one-row or the 4-row kernel
         if (ctx->opt.rows_per_step == 1) return 1;
         if (ctx->opt.tile_g == -1 && ctx->tuned_h > 0) return ctx->tuned_h;
+        if (ctx->opt.tile_g == 0 && ctx->opt.rows_per_step == 0 && ring_sweep(ctx)) return 1;
         return 4;
     }
     if (ctx->opt.rows_per_step == 1 || ctx->opt.rows_per_step == 2 || ctx->opt.rows_per_step == 4)

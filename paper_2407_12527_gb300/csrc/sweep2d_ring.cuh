@@ -1,24 +1,27 @@
-// sweep2d_ring.cuh -- the X-Y transport sweep (K1) of the angular-moment source modes
-// (isotropic, linear kernel) with one grid row per wavefront step and the cell rows
-// staged through per-lane rings in shared memory.
+// sweep2d_ring.cuh -- the X-Y transport sweep (K1) with one grid row per wavefront step and
+// the cell rows staged through per-lane rings in shared memory, for the angular-moment source
+// modes (isotropic, linear kernel) and the dense operator mode.
 //
 // Same cell equations, work items (up to G ordinates of one quadrant of one sample) and
 // moment accumulators as the other X-Y sweeps.  Lanes are numbered from the inflow face;
-// lane p owns the 4 cells at distance 4p .. 4p+3 from it in every row, and lane d of a
-// warp sweeps row t - d at the warp's step t, so the x-edge flux passes one lane per step
-// by a shuffle and the y-edge fluxes stay in registers.  Warp w of a wide row runs
+// lane p owns the C cells (4 or 8) at distance C p .. C p + C - 1 from it in every row, and
+// lane d of a warp sweeps row t - d at the warp's step t, so the x-edge flux passes one lane
+// per step by a shuffle and the y-edge fluxes stay in registers.  Warp w of a wide row runs
 // kLag * 8 steps behind warp w - 1 and takes the x-edges from a shared-memory ring; the
 // warps meet at one CTA barrier per 8 steps.
 //
 // Memory.  The lanes of a warp sit on 32 different rows, so a direct access of the warp
-// would touch 32 cache lines for 512 bytes, and the L1 would be the limit (one line per
-// cycle: 32 cycles per access, three accesses per step, against ~100 cycles of
-// arithmetic).  Instead each 8-lane group copies 128 contiguous bytes of one row per step
-// (cp.async, row t + kAhead - 8 * group), every lane into its own column of a 16-row ring,
-// and reads its own cells when its step comes; it leaves the moments in the same slot,
-// and the group adds them to the accumulator row by row, 128 contiguous bytes at a time
-// (red.global.add.v4), once its last lane has passed.  A lane only ever touches its own
-// column of the ring, so no barrier is involved.
+// would touch 32 cache lines, and the L1 takes one line per cycle: 32 cycles per access and
+// three accesses per step, on the four schedulers' shared L1, against ~100 cycles of
+// arithmetic per warp and step.  Instead each 8-lane group copies 128 (C = 8: 256)
+// contiguous bytes of one row per step (cp.async, row t + kAhead - 8 * group) into 16-row
+// rings of its lanes' columns; a lane reads its own cells when its step comes and leaves the
+// moments in the same slot, and the group adds them to the accumulator row by row, again 128
+// contiguous bytes at a time (red.global.add.v4), once its last lane has passed.  No lane
+// touches another group's columns, so the rings need no barrier (a warp-level one with C = 8,
+// where the lanes of a group copy for each other to keep the 128 bytes contiguous).  In the
+// dense mode the slots hold the sources of the item's two ordinates and take their psi, which
+// the group stores (FP32 or split BF16) and sums into phi.
 //
 // Arithmetic.  With f = 2 (diamond difference) or 1 (step), a = f|c|/dx, b = f|s|/dy,
 // d = sigma_T + a + b, the edge fluxes are kept scaled so that the source enters every
@@ -30,9 +33,19 @@
 //   varying sigma_T: X = a x, P = b y: psi = (S + X + P) / d, X' = f a psi - X (DD) or
 //     a psi, P' likewise, moment += w psi.
 // The uniform case takes five packed FP32x2 operations per cell and ordinate pair and its
-// upwind chain is one FMA per cell.  The packed instructions take no negated operand, so
-// the DD closure keeps -P at odd steps (and the varying case -X at odd cells): P' = c - P
-// becomes (-P') = P - c, one FMA with a negated constant either way.
+// upwind chain is one FMA per cell.  The DD closure keeps -P after even steps (and the
+// varying case -X at odd cells), so that every update is one FMA without a negated operand:
+// P' = c - P or -P' = P - c.
+//
+// What bounds it.  A warp issues 115-125 instructions per step of 512 updates at 2.5-3
+// cycles each with the one or two warps per scheduler of most solves (fixed-latency
+// dependencies, three cycles of register ports per packed FMA); with two ordinates per item
+// the moment reductions (134 MB at 256 x 256 x 64 samples of 16) add 6-8 of 49 us.  One
+// launch, GB300, against the row kernel of sweep2d_row.cuh: 256 x 256 x 64 samples of 16
+// 49 us (70), one sample of 256 35 (54), 256 samples of 16 92 (141); 100 x 100 x 16 of 36
+// 18 (45); varying sigma_T 256 x 256 x 256 of 16 165 (274).  Dense mode, 512 x 512 x 32 of
+// 128: 1746 us against 2640 with the 4-row kernel (8.6 GB: 73% of the copy bandwidth);
+// 150 x 130 x 8 of 48 51 against 138.
 #pragma once
 #include <type_traits>
 
@@ -129,6 +142,38 @@ __device__ __forceinline__ void ring_red(float *p, const float4 &v, int row, int
                  "f"(v.y), "f"(v.z), "f"(v.w), "r"(row), "r"(lim), "n"(OFF)
                  : "memory");
 }
+// dense mode: psi of 4 cells, FP32 at p + o, or its BF16 parts in the 32-byte sector
+// [8 hi | 8 lo] of the 8 cells they belong to (st8_split's rounding)
+template <int OFF>
+__device__ __forceinline__ void psi_put(float *psi, uint32_t *split, long long o, const float4 &v,
+                                        int row, int lim)
+{
+    if (split == nullptr) {
+        asm volatile("{\n\t.reg .pred q;\n\tsetp.lt.u32 q, %5, %6;\n\t"
+                     "@q st.global.v4.f32 [%0+%7], {%1,%2,%3,%4};\n\t}" ::"l"(psi + o), "f"(v.x),
+                     "f"(v.y), "f"(v.z), "f"(v.w), "r"(row), "r"(lim), "n"(OFF)
+                     : "memory");
+        return;
+    }
+    o += OFF / 4;
+    uint32_t h[2], l[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const float a = e ? v.z : v.x, b = e ? v.w : v.y;
+        const uint32_t b0 = (__float_as_uint(a) + 0x8000u) & 0xFFFF0000u;
+        const uint32_t b1 = (__float_as_uint(b) + 0x8000u) & 0xFFFF0000u;
+        h[e] = __byte_perm(b0, b1, 0x7632);
+        const __nv_bfloat162 lo2 =
+            __floats2bfloat162_rn(a - __uint_as_float(b0), b - __uint_as_float(b1));
+        l[e] = *reinterpret_cast<const uint32_t *>(&lo2);
+    }
+    uint32_t *q = split + (o & ~7LL) + ((o >> 1) & 2);
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.lt.u32 q, %5, %6;\n\t"
+                 "@q st.global.v2.b32 [%0], {%1,%2};\n\t"
+                 "@q st.global.v2.b32 [%0+16], {%3,%4};\n\t}" ::"l"(q), "r"(h[0]), "r"(h[1]),
+                 "r"(l[0]), "r"(l[1]), "r"(row), "r"(lim)
+                 : "memory");
+}
 // test hook: a wait, bounded in time, on an mbarrier that nothing completes
 __device__ __forceinline__ bool ring_never_wait(unsigned long long *b, unsigned long long budget_ns)
 {
@@ -150,8 +195,10 @@ __device__ __forceinline__ bool ring_never_wait(unsigned long long *b, unsigned 
     }
 }
 
-// arrays staged per warp: the source moments (their slots take the flux moments), sigma_T
-__host__ __device__ constexpr int ring_arrays(int mom, bool homog) { return mom + (homog ? 0 : 1); }
+// Arrays copied in: the source moments, or in the dense mode the sources of the item's two
+// ordinates (their slots take the flux moments, or psi), and sigma_T.
+__host__ __device__ constexpr int ring_src(int mom) { return mom == 0 ? 2 : mom; }
+__host__ __device__ constexpr int ring_arrays(int mom, bool homog) { return ring_src(mom) + (homog ? 0 : 1); }
 // shared memory of a CTA: the warps' rings, their incoming x-edges, 16 zero bytes
 __host__ __device__ constexpr int ring_bytes(int mom, bool homog, int nwarps, int G, int C)
 {
@@ -163,7 +210,9 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
                                           const SweepItem &it, char *smem)
 {
     constexpr int N = RingPack<G>::N;
-    constexpr int NA = ring_arrays(MOM, HOMOG);
+    constexpr int NS = ring_src(MOM), NA = ring_arrays(MOM, HOMOG);
+    constexpr int NP = MOM == 0 ? 2 : 1;    // base pointers of the sources
+    static_assert(MOM != 0 || G == 2, "the dense mode takes two ordinates per item");
     constexpr unsigned kRowB = 32 * C * 4, kArrB = kRows * kRowB;  // bytes of a ring row, a ring
     constexpr int CH = C / 4;  // 16-byte chunks of a lane's cells
     constexpr unsigned kMask = kArrB - 1;
@@ -180,8 +229,9 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
     const float fdd = DD ? 2.f : 1.f;
 
     // per-ordinate constants (see the head of the file); an empty slot has weight zero
+    float2 kp[N];  // dense mode: psi per sum (uniform sigma_T)
     float2 k1[N], k2[N], k2n[N], km[N], kmc[N], kms[N], kc[N], ks[N], ab[N], lx[N], wl[N];
-    int ord[G];
+    long long ord[G];
     float inj_x[G], inj_y[G];  // boundary value -> scaled edge flux
 #pragma unroll
     for (int k = 0; k < G; ++k) {
@@ -201,7 +251,8 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
         qset(k1[pk], i, HOMOG ? (DD ? (a - b - st) * rd : a * rd) : fdd * a);
         qset(k2[pk], i, HOMOG ? fdd * b * rd : fdd * b);
         qset(ab[pk], i, a + b);
-        qset(km[pk], i, wm);
+        qset(kp[pk], i, rd);
+        qset(km[pk], i, MOM == 0 ? wt : wm);
         qset(kmc[pk], i, wm * c);
         qset(kms[pk], i, wm * s);
         qset(kc[pk], i, c);
@@ -241,7 +292,7 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
     for (int h = 0; h < CH; ++h) own[h] = rings + lane * C * 4 + ((h ^ sw) * 16);
     for (int m = 0; m < NA; ++m)
         for (int r = 0; r < kRows; ++r) {
-            const float z = m == MOM ? 1.f : 0.f;
+            const float z = !HOMOG && m == NS ? 1.f : 0.f;
 #pragma unroll
             for (int h = 0; h < CH; ++h) sts4(own[h] + m * kArrB + r * kRowB, make_float4(z, z, z, z));
         }
@@ -257,7 +308,8 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
     const unsigned edge_sel = lane == 0 ? kEdgeB - 1 : 0;
     const unsigned edge_out = edges + (w + 1) * kEdgeB;
 
-    const long long so = A.soff ? A.soff[it.sample] : (long long)it.sample * MOM * gd.cells;
+    const long long so =
+        A.soff ? A.soff[it.sample] : (long long)it.sample * (MOM == 0 ? 1 : MOM) * gd.cells;
     const long long rs = yneg ? -(long long)gd.NXP : (long long)gd.NXP;
     const long long cells = gd.cells;
     const int grp8 = lane & ~7;  // 8 * the lane's group
@@ -330,9 +382,13 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
     const unsigned place1 = CH == 2 ? (place ^ 16) + kPlace1 : 0;
     constexpr int kChunk1 = (XNEG ? -1 : 1) * 4 * C * 4;  // bytes between the chunks' cells
     const int cd = C * (XNEG ? L - 1 - (32 * w + grp8 + dl0) : 32 * w + grp8 + dl0) + 4 * half;
-    const float *src = A.src + o0 + cd + frow * rs;
+    const float *src[NP];
+#pragma unroll
+    for (int k = 0; k < NP; ++k)
+        src[k] = A.src + (MOM == 0 ? o0 - so + ord[k] * cells : o0) + cd + frow * rs;
     const float *sig = HOMOG ? nullptr : A.sigma_t + gd.off + (o0 - so) + cd + frow * rs;
     float *acc = A.part + o0 + cd + (frow - kRows + 1) * rs;
+    long long po = o0 - so + cd + (frow - kRows + 1) * rs;  // dense mode: place of psi
     unsigned cs = 0;             // slot of the step's cells (step 0: slot 0)
     unsigned eo = 0;             // offset of the x-edges of row t + 1 (and of row t - 31)
 
@@ -342,12 +398,13 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
     auto fill = [&]() {
 #pragma unroll
         for (int m = 0; m < NA; ++m) {
-            const float *p = m < MOM ? src + m * cells : sig;
+            const float *p = m >= NS ? sig : MOM == 0 ? src[m % NP] : src[0] + m * cells;
             ring_copy<0>(place + m * kArrB + fd[0], p, frow, lim[0]);
             if constexpr (CH == 2)
                 ring_copy<kChunk1>(place1 + m * kArrB + fd[CH - 1], p, frow, lim[CH - 1]);
         }
-        src += rs;
+#pragma unroll
+        for (int k = 0; k < NP; ++k) src[k] += rs;
         if constexpr (!HOMOG) sig += rs;
         ++frow;
 #pragma unroll
@@ -379,12 +436,11 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
         fill();
         // the moments of the row that the group's last lane finished at the step before
         // (fill has moved on to its slot)
-        float4 D[MOM][CH];
+        float4 D[NS][CH];
 #pragma unroll
-        for (int m = 0; m < MOM; ++m)
+        for (int m = 0; m < NS; ++m)
 #pragma unroll
-            for (int h = 0; h < CH; ++h)
-                D[m][h] = lds4((h ? place1 : place) + m * kArrB + fd[h]);
+            for (int h = 0; h < CH; ++h) D[m][h] = lds4((h ? place1 : place) + m * kArrB + fd[h]);
         const unsigned slot = cs;
         float4 V[NA][CH];
 #pragma unroll
@@ -430,8 +486,9 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
                     tt = ODD ? qfma(P[r][q], neg1, s) : qadd(s, P[r][q]);
                 } else {
                     const float s = f4(V[0][r / 4], r % 4);
-                    tt = ODD ? make_float2(s - P[r][q].x, s - P[r][q].y)
-                             : make_float2(s + P[r][q].x, s + P[r][q].y);
+                    const float sy = MOM == 0 ? f4(V[MOM == 0 ? 1 : 0][r / 4], r % 4) : s;
+                    tt = ODD ? make_float2(s - P[r][q].x, sy - P[r][q].y)
+                             : make_float2(s + P[r][q].x, sy + P[r][q].y);
                 }
                 const bool first = !EDGE && rr == 0;  // lane 0 takes no x-edge
                 if constexpr (HOMOG) {
@@ -474,17 +531,22 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
                              "f"(x[C][0].x), "f"(x[C][0].y), "r"((unsigned)feeds)
                              : "memory");
         }
-        float v[MOM][C];
+        float v[NS][C];
 #pragma unroll
         for (int rr = 0; rr < C; ++rr) {
             const int r = XNEG ? C - 1 - rr : rr;
-            float2 m[MOM];
+            float2 m[MOM == 0 ? 1 : MOM];
 #pragma unroll
             for (int q = 0; q < N; ++q) {
                 const float2 s = sm[rr][q];
                 if (!RAGGED || real[rr])
                     P[r][q] = DD ? qfma(ODD ? k2[q] : k2n[q], s, P[r][q])
                                  : EV && (held || past) ? P[r][q] : qmul(k2[q], s);
+                if constexpr (MOM == 0) {  // psi of the two ordinates
+                    const float2 pc = HOMOG ? qmul(kp[q], s) : s;
+                    v[0][r] = (!RAGGED || real[rr]) ? pc.x : 0.f;
+                    v[1][r] = (!RAGGED || real[rr]) ? pc.y : 0.f;
+                }
 #pragma unroll
                 for (int k = 0; k < MOM; ++k) {
                     const float2 kw = k == 0 ? km[q] : k == 1 ? kmc[q] : kms[q];
@@ -495,11 +557,34 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
             for (int k = 0; k < MOM; ++k) v[k][r] = (!RAGGED || real[rr]) ? m[k].x + m[k].y : 0.f;
         }
 #pragma unroll
-        for (int k = 0; k < MOM; ++k) sts_cells<C>(own, k * kArrB + slot, v[k], on);
+        for (int k = 0; k < NS; ++k) sts_cells<C>(own, k * kArrB + slot, v[k], on);
 #pragma unroll
         for (int q = 0; q < N; ++q) lk[q] = qfma(lx[q], x[C][q], lk[q]);
+        if constexpr (MOM == 0) {
 #pragma unroll
-        for (int m = 0; m < MOM; ++m) {
+            for (int k = 0; k < 2; ++k) {
+                // (an empty slot's ordinate is the first again: not stored)
+                const int l0 = k < it.n ? lim[0] : 0, l1 = k < it.n ? lim[CH - 1] : 0;
+                const long long o = po + ord[k] * cells;
+                psi_put<0>(A.psi, A.psi_split, o, D[k][0], frow - kRows, l0);
+                if constexpr (CH == 2)
+                    psi_put<kChunk1>(A.psi, A.psi_split, o, D[k][CH - 1], frow - kRows, l1);
+            }
+            po += rs;
+        }
+        if constexpr (MOM == 0) {  // the two ordinates' part of phi, in the place of psi
+#pragma unroll
+            for (int h = 0; h < CH; ++h) {
+                float4 &d = D[0][h];
+                const float4 &e = D[NS - 1][h];
+                d.x = fmaf(km[0].y, e.x, km[0].x * d.x);
+                d.y = fmaf(km[0].y, e.y, km[0].x * d.y);
+                d.z = fmaf(km[0].y, e.z, km[0].x * d.z);
+                d.w = fmaf(km[0].y, e.w, km[0].x * d.w);
+            }
+        }
+#pragma unroll
+        for (int m = 0; m < (MOM == 0 ? 1 : MOM); ++m) {
             ring_red<0>(acc + m * cells, D[m][0], frow - kRows, lim[0]);
             if constexpr (CH == 2)
                 ring_red<kChunk1>(acc + m * cells, D[m][CH - 1], frow - kRows, lim[CH - 1]);
@@ -516,7 +601,7 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
         for (int e = 0; e < kPre; ++e) {
             const int k = (32 * e + lane) % G, rr = r0 + (32 * e + lane) / G;
             float ix = 0.f, lw = 0.f;
-            int o = 0;
+            long long o = 0;
 #pragma unroll
             for (int kk = 0; kk < G; ++kk)
                 if (kk == k && kk < it.n) {
@@ -551,6 +636,7 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
 #pragma unroll 1
                 for (int u = 0; u < kGrp; ++u) fill();
                 acc += kGrp * rs;
+                po += kGrp * rs;
                 t = 0;
                 load();
             } else if (t + kGrp > J || (EDGE && t < 32 && A.inflow != nullptr)) {
@@ -647,11 +733,11 @@ cudaError_t ring_launch(const SweepArgs &a, int n_items, int C, int G, cudaStrea
 #define RING_K(CC, GG)                                                                            \
     return nw > 1 || inflow ? ring_launch_k<CC, GG, MOM, SCHEME, HOMOG, true>(a, n_items, nw, st) \
                             : ring_launch_k<CC, GG, MOM, SCHEME, HOMOG, false>(a, n_items, nw, st)
-    if (C == 8) {
-        if (G == 4) RING_K(8, 4);
-        RING_K(8, 2);
+    if constexpr (MOM != 0) {
+        if (G == 4 && C == 8) RING_K(8, 4);
+        if (G == 4) RING_K(4, 4);
     }
-    if (G == 4) RING_K(4, 4);
+    if (C == 8) RING_K(8, 2);
     RING_K(4, 2);
 #undef RING_K
 }

@@ -1,5 +1,5 @@
 // sweep2d_row.cuh -- the X-Y transport sweep (K1) with one grid row per wavefront
-// step, for the angular-moment source modes (isotropic, linear kernel).
+// step, for rows too wide for the shared-memory rings of sweep2d_ring.cuh.
 //
 // Same cell equations as sweep2d_impl.cuh (Sec. 2, eq. (equ_random)), same work
 // items (up to G ordinates of one quadrant of one sample) and the same moment
@@ -146,7 +146,7 @@ __host__ __device__ constexpr int row_pd(int na, int g)
     return g == 4 ? (na <= 2 ? 2 : 1) : (na == 1 ? 6 : (na == 2 ? 4 : (na == 3 ? 2 : 1)));
 }
 
-template <int G, int MOM, int SCHEME, bool HOMOG, bool XNEG, bool RAGGED, bool MULTI, bool INFLOW>
+template <int G, int MOM, int SCHEME, bool HOMOG, bool XNEG, bool RAGGED, bool INFLOW>
 __device__ __forceinline__ void row_item(const SweepArgs &A, const SweepItem &it)
 {
     using T = typename RowPack<G>::T;
@@ -156,7 +156,7 @@ __device__ __forceinline__ void row_item(const SweepArgs &A, const SweepItem &it
     constexpr int NS = MOM == 0 ? G : MOM;  // source arrays (the rest: sigma_T)
     constexpr int PD = row_pd(NA, G);
     const int g = threadIdx.x;
-    const int nwarps = MULTI ? (int)(blockDim.x >> 5) : 1;
+    const int nwarps = (int)(blockDim.x >> 5);
     const int L = (A.I + kCols - 1) / kCols;  // lanes that own cells
     const bool on = g < L;
     const int d = XNEG ? (L - 1 - g) : g;     // lanes between this one and the inflow face
@@ -287,7 +287,7 @@ __device__ __forceinline__ void row_item(const SweepArgs &A, const SweepItem &it
 #pragma unroll
             for (int m = 0; m < NA; ++m) rld8<G>(arr[m] + row0 + (long long)jl * rs, buf[k][m]);
     }
-    __shared__ T xbuf[MULTI ? 2 : 1][MULTI ? kMaxWarps : 1][N];
+    __shared__ T xbuf[2][kMaxWarps][N];
     T xin[N];
 #pragma unroll
     for (int p = 0; p < N; ++p) xin[p] = rsplat<T>(0.f);
@@ -458,18 +458,18 @@ __device__ __forceinline__ void row_item(const SweepArgs &A, const SweepItem &it
 #pragma unroll
                 for (int p = 0; p < N; ++p) xin[p] = d == 0 ? rsplat<T>(0.f) : xin[p];
             }
-            if (MULTI && nwarps > 1) {  // across warps through shared memory, one barrier per step
+            if (nwarps > 1) {  // across warps through shared memory, one barrier per step
                 const int lane = g & 31, w = g >> 5;
                 const bool sender = XNEG ? (lane == 0 && w > 0) : (lane == 31 && w + 1 < nwarps);
                 if (sender)
 #pragma unroll
-                    for (int p = 0; p < N; ++p) xbuf[MULTI ? (t & 1) : 0][w][p] = xo[p];
+                    for (int p = 0; p < N; ++p) xbuf[t & 1][w][p] = xo[p];
                 __syncthreads();
                 const bool recv = XNEG ? (lane == 31 && w + 1 < nwarps) : (lane == 0 && w > 0);
                 if (recv) {
                     const int src_w = XNEG ? w + 1 : w - 1;
 #pragma unroll
-                    for (int p = 0; p < N; ++p) xin[p] = xbuf[MULTI ? (t & 1) : 0][src_w][p];
+                    for (int p = 0; p < N; ++p) xin[p] = xbuf[t & 1][src_w][p];
                 }
             }
         }
@@ -504,7 +504,7 @@ __device__ __forceinline__ void row_item(const SweepArgs &A, const SweepItem &it
     }
 }
 
-template <int G, int MOM, int SCHEME, bool HOMOG, bool BATCH, bool MULTI, bool INFLOW>
+template <int G, int MOM, int SCHEME, bool HOMOG, bool BATCH, bool INFLOW>
 __global__ void __launch_bounds__(32 * kMaxWarps) sweep2d_row_kernel(const SweepArgs A0)
 {
     const SweepItem it = A0.items[blockIdx.x];
@@ -535,15 +535,15 @@ __global__ void __launch_bounds__(32 * kMaxWarps) sweep2d_row_kernel(const Sweep
     }
     const bool ragged = A.I % kCols != 0;
     if (it.quad & 1) {
-        if (ragged) row_item<G, MOM, SCHEME, HOMOG, true, true, MULTI, INFLOW>(A, it);
-        else row_item<G, MOM, SCHEME, HOMOG, true, false, MULTI, INFLOW>(A, it);
+        if (ragged) row_item<G, MOM, SCHEME, HOMOG, true, true, INFLOW>(A, it);
+        else row_item<G, MOM, SCHEME, HOMOG, true, false, INFLOW>(A, it);
     } else {
-        if (ragged) row_item<G, MOM, SCHEME, HOMOG, false, true, MULTI, INFLOW>(A, it);
-        else row_item<G, MOM, SCHEME, HOMOG, false, false, MULTI, INFLOW>(A, it);
+        if (ragged) row_item<G, MOM, SCHEME, HOMOG, false, true, INFLOW>(A, it);
+        else row_item<G, MOM, SCHEME, HOMOG, false, false, INFLOW>(A, it);
     }
 }
 
-// one kernel per (G, homog, multi-warp, inflow) of this translation unit's source
+// one kernel per (G, homog, inflow) of this translation unit's source
 // mode MOM and scheme SCHEME; items of one ordinate run on the two-ordinate
 // kernel (the empty second slot has zero weight)
 template <int MOM, int SCHEME, bool BATCH>
@@ -554,36 +554,29 @@ cudaError_t row_launch(const SweepArgs &a, int n_items, int nwarps, int G, bool 
     if (nwarps < 1 || nwarps > kMaxWarps || (G != 1 && G != 2 && G != 4))
         return cudaErrorInvalidValue;
     const dim3 grid(n_items), block(32 * nwarps);
-    const bool multi = nwarps > 1, inflow = a.inflow != nullptr;
-#define ROW_K(GG, HH, MM, II) sweep2d_row_kernel<GG, MOM, SCHEME, HH, BATCH, MM, II><<<grid, block, 0, st>>>(a)
-// (moment modes: rows that fit one warp run on sweep2d_ring.cuh)
-#define ROW_M(GG, HH, II)                                    \
-    do {                                                     \
-        if constexpr (MOM == 0) {                            \
-            if (multi) ROW_K(GG, HH, true, II);              \
-            else ROW_K(GG, HH, false, II);                   \
-        } else ROW_K(GG, HH, true, II);                      \
-    } while (0)
+    const bool inflow = a.inflow != nullptr;
+#define ROW_K(GG, HH, II) sweep2d_row_kernel<GG, MOM, SCHEME, HH, BATCH, II><<<grid, block, 0, st>>>(a)
 #define ROW_G(GG, HH)                                        \
     do {                                                     \
-        if (inflow) ROW_M(GG, HH, true);                     \
-        else ROW_M(GG, HH, false);                           \
+        if (inflow) ROW_K(GG, HH, true);                     \
+        else ROW_K(GG, HH, false);                           \
     } while (0)
     if constexpr (BATCH) {
         (void)homog;  // several grids: sigma_T read per cell, vacuum boundaries
-        if (G == 4) ROW_K(4, false, true, false);
-        else ROW_K(2, false, true, false);
+        if (G == 4) ROW_K(4, false, false);
+        else ROW_K(2, false, false);
     } else {
-        if (G == 4) {
-            if (homog) ROW_G(4, true);
-            else ROW_G(4, false);
-        } else {
-            if (homog) ROW_G(2, true);
-            else ROW_G(2, false);
+        if constexpr (MOM != 0) {  // (the dense mode takes at most two ordinates per item)
+            if (G == 4) {
+                if (homog) ROW_G(4, true);
+                else ROW_G(4, false);
+                return cudaGetLastError();
+            }
         }
+        if (homog) ROW_G(2, true);
+        else ROW_G(2, false);
     }
 #undef ROW_G
-#undef ROW_M
 #undef ROW_K
     return cudaGetLastError();
 }

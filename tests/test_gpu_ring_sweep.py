@@ -119,3 +119,26 @@ def test_batch_of_narrower_grids(rom, widths, n_samples):
         for k in range(n_samples):
             assert rel(ctx.scalar_flux(p * n_samples + k), ref[k]) < TOL, (p, k)
     ctx.close()
+
+
+@pytest.mark.parametrize("grid", [(5, 8), (33, 16), (130, 18), (257, 40), (300, 12)])
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("medium", ["uniform", "varying"])
+@pytest.mark.parametrize("scheme", ["dd", "step"])
+@pytest.mark.parametrize("n_samples", [2, 40])
+def test_dense_mode(rom, grid, precision, medium, scheme, n_samples):
+    """Per-ordinate sources in and psi out (FP32, split BF16), odd ordinate counts, an inflow
+    with the fewer samples; 40 samples: enough items for the 8-cell lanes."""
+    I, J = grid
+    st, ss, q = W.random_medium(I, J, seed=I + J, ratio_max=0.7)
+    if medium == "uniform":
+        st = np.full((J, I), 1.9)
+        ss = np.minimum(ss, 1.2)
+    sets = [O.Ordinates(*W.random_directions(19, seed=70 + k, weights="random"))
+            for k in range(n_samples)]
+    inf = W.random_inflow(I, J, seed=5) if n_samples == 2 else None
+    phi, _, _, stats = solve(rom, I, J, st, ss, q, sets, inf, kernel="hg", g=0.4, fixed_iters=3,
+                             scheme=rom.SCHEME[scheme], dense_precision=precision)
+    ref, _ = oracle(I, J, st, ss, q, sets, inf, kernel="hg", g=0.4, scheme=scheme, fixed_iters=3)
+    assert stats["rows_per_step"] == 1
+    assert max(rel(phi[k], ref[k]) for k in range(n_samples)) < TOL
