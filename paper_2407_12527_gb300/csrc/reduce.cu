@@ -333,55 +333,64 @@ __global__ void __launch_bounds__(256) finalize_kernel(const FinalizeArgs A)
     }
 }
 
-__global__ void init_checks_kernel(int S, double *dprev, int *grow, double *leak, double *bal,
-                                   double *leak_out, double *phimin, double *sums, int *minkey)
-{
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= S) return;
-    dprev[s] = (double)INFINITY;
-    grow[s] = 0;
-    leak[s] = 0.0;
-    bal[s] = (double)NAN;
-    leak_out[s] = (double)NAN;
-    phimin[s] = (double)NAN;
-#pragma unroll
-    for (int k = 0; k < kNP; ++k) sums[(long long)s * kNP + k] = 0.0;
-    minkey[s] = 0x7FFFFFFF;
-}
-
+// one warp per sample
 __global__ void ordsum_kernel(const double *c, const double *s, const double *w,
                               const long long *ord_off, const int *M, int S, double *out)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    const int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (k >= S) return;
     double sw = 0.0, swc = 0.0, sws = 0.0;
-    for (long long o = ord_off[k]; o < ord_off[k] + M[k]; ++o) {
+    for (long long o = ord_off[k] + lane; o < ord_off[k] + M[k]; o += 32) {
         sw += w[o];
         swc += w[o] * c[o];
         sws += w[o] * s[o];
     }
-    out[3 * k] = sw;
-    out[3 * k + 1] = swc;
-    out[3 * k + 2] = sws;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        sw += __shfl_xor_sync(0xffffffffu, sw, d);
+        swc += __shfl_xor_sync(0xffffffffu, swc, d);
+        sws += __shfl_xor_sync(0xffffffffu, sws, d);
+    }
+    if (lane == 0) {
+        out[3 * k] = sw;
+        out[3 * k + 1] = swc;
+        out[3 * k + 2] = sws;
+    }
 }
 
 __global__ void init_state_kernel(int S, int MOM, long long cells, const float *q, float *phi,
-                                  float *src, int *active, int *iters, int *flags, double *resid)
+                                  float *src, float *part, InitState is)
 {
-    const long long n = (long long)S * MOM * cells;
-    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n;
-         v += (long long)gridDim.x * blockDim.x) {
-        const long long cell = v % cells;
-        const int m = (int)((v / cells) % MOM);
-        phi[v] = 0.f;
-        if (src) src[v] = m == 0 ? q[cell] : 0.f;  // psi^0 = 0: the first source is q
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    const long long n4 = cells / 4;  // (cells is a multiple of 8)
+    for (long long sm = blockIdx.y; sm < (long long)S * MOM; sm += gridDim.y) {
+        float4 *p = (float4 *)(phi + sm * cells), *a = (float4 *)(part + sm * cells);
+        float4 *f = (float4 *)(src + sm * cells);
+        for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n4;
+             v += (long long)gridDim.x * blockDim.x) {
+            p[v] = zero;
+            if (part) a[v] = zero;
+            // psi^0 = 0: the first source is q
+            if (src) f[v] = sm % MOM == 0 ? ((const float4 *)q)[v] : zero;
+        }
     }
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < S) {
-        active[t] = 1;
-        iters[t] = 0;
-        flags[t] = 0;
-        resid[t] = (double)INFINITY;
+    if (blockIdx.y > 0) return;
+    const int t0 = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t0 < 4) is.err[t0] = 0;
+    for (long long t = t0; t < S; t += (long long)gridDim.x * blockDim.x) {
+        is.active[t] = 1;
+        is.iters[t] = 0;
+        is.flags[t] = 0;
+        is.resid[t] = (double)INFINITY;
+        is.dprev[t] = (double)INFINITY;
+        is.grow[t] = 0;
+        is.leak[t] = 0.0;
+        is.bal[t] = (double)NAN;
+        is.leak_out[t] = (double)NAN;
+        is.phimin[t] = (double)NAN;
+#pragma unroll
+        for (int k = 0; k < kNP; ++k) is.sums[t * kNP + k] = 0.0;
+        is.minkey[t] = 0x7FFFFFFF;
     }
 }
 
@@ -529,14 +538,12 @@ cudaError_t launch_finalize(const FinalizeArgs &a, cudaStream_t st)
 }
 
 cudaError_t launch_init_state(int S, int MOM, long long cells, const float *q, float *phi,
-                              float *src, int *active, int *iters, int *flags, double *resid,
-                              cudaStream_t st)
+                              float *src, float *part, const InitState &is, cudaStream_t st)
 {
-    long long n = (long long)S * MOM * cells;
-    if (n < S) n = S;
-    int b = blocks_for(n, 256);
-    if ((long long)b * 256 < S) b = (S + 255) / 256;
-    init_state_kernel<<<b, 256, 0, st>>>(S, MOM, cells, q, phi, src, active, iters, flags, resid);
+    const long long bx = std::min(std::max((cells / 4 + 255) / 256, 1LL), 256LL);
+    const long long by = std::min((long long)S * MOM, std::max(1LL, 8192 / bx));
+    init_state_kernel<<<dim3((unsigned)bx, (unsigned)by), 256, 0, st>>>(S, MOM, cells, q, phi, src,
+                                                                       part, is);
     return cudaGetLastError();
 }
 
@@ -578,16 +585,7 @@ cudaError_t launch_ordsum(const double *c, const double *s, const double *w,
                           const long long *ord_off, const int *M, int S, double *out,
                           cudaStream_t st)
 {
-    ordsum_kernel<<<(S + 127) / 128, 128, 0, st>>>(c, s, w, ord_off, M, S, out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_init_checks(int S, double *dprev, int *grow, double *leak, double *bal,
-                               double *leak_out, double *phimin, double *sums, int *minkey,
-                               cudaStream_t st)
-{
-    init_checks_kernel<<<(S + 255) / 256, 256, 0, st>>>(S, dprev, grow, leak, bal, leak_out,
-                                                        phimin, sums, minkey);
+    ordsum_kernel<<<(S + 3) / 4, 128, 0, st>>>(c, s, w, ord_off, M, S, out);
     return cudaGetLastError();
 }
 

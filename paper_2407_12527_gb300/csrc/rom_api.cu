@@ -105,9 +105,14 @@ struct rom_ctx {
     long long state_floats = 0;      // floats of one per-sample state array (all samples)
     long long max_cells = 0;         // largest grid's J * NXP
     DevBuf gdesc, sgrid_dev, soff_dev, sdA_dev;
-    // per-sample divergence and balance state: dprev, grow, leak (added by the
-    // sweep), bal / leak_out / phimin (last sweep); the X-Y sweep's wait flag
-    DevBuf dprev, grow, leak, bal, leak_out, phimin, sweep_err;
+    // per-sample divergence and balance state: dprev, grow, leak (added by the sweep)
+    DevBuf dprev, grow, leak;
+    // What a solve reports, in one device block and its pinned host copy, so that one copy
+    // brings it back: [S] resid, bal, leak_out, phimin (of the last sweep; FP64), [S] iters,
+    // flags, and the error words of the X-Y sweep, the 3D sweep and the tensor-core product.
+    DevBuf result;
+    unsigned char *h_result = nullptr;
+    size_t h_result_cap = 0;
     std::vector<double> h_bal, h_leak, h_phimin;
     std::vector<SweepItem> items;
     DevBuf items_dev;
@@ -115,14 +120,14 @@ struct rom_ctx {
     size_t h_stage_cap = 0;
     // 3D: CTA item lists (one octant each) and the tile hand-off buffers
     std::vector<int> cta_begin, cta_list;
-    DevBuf cta_begin_dev, cta_list_dev, xface, yface, err3;
+    DevBuf cta_begin_dev, cta_list_dev, xface, yface;
     // 3D diagonal storage: sigma_T [2], source and flux [2][S], sigma_S and q (family 0);
     // phi is kept in family 0 as well ([S][sk.cells])
     DevBuf sig3, src3, acc3, ss3, q3;
     int n_ctas3 = 0, nwarps3 = 1, n_tx = 1, n_ty = 1;
 
     // dense scattering operator (mode 0); tensor-core variant: split BF16 psi and A
-    DevBuf psi, src_ord, Amat, dtab, psi_split, a_hi, a_lo, tc_err;
+    DevBuf psi, src_ord, Amat, dtab, psi_split, a_hi, a_lo;
     bool pmat_dirty = true;
     romk::DenseTcMaps tc_maps;
     const void *tc_map_ptrs[3] = {nullptr, nullptr, nullptr};
@@ -132,7 +137,7 @@ struct rom_ctx {
     // iteration state
     int MOM = 1;  // 1 isotropic moments, 3 linear moments, 0 dense operator
     int chunks = 1;
-    DevBuf phi, src, part, sums, minkey, active, iters, flags, resid, n_active, avg, sum, tmp;
+    DevBuf phi, src, part, sums, minkey, active, n_active, avg, sum, tmp;
     bool solved = false;
     std::vector<int> h_iters;
     std::vector<double> h_resid;
@@ -203,6 +208,40 @@ int ensure_host_stage(rom_ctx *ctx, size_t bytes)
     }
     ctx->h_stage = (float *)p;
     ctx->h_stage_cap = bytes;
+    return ROM_OK;
+}
+
+// the result block of a solve (rom_ctx::result) at a base address, device or host
+struct Result {
+    double *resid, *bal, *leak_out, *phimin;
+    int *iters, *flags, *err;
+};
+size_t result_bytes(const rom_ctx *ctx)
+{
+    return (size_t)ctx->S * (4 * sizeof(double) + 2 * sizeof(int)) + 4 * sizeof(int);
+}
+Result result_view(const rom_ctx *ctx, void *base)
+{
+    const size_t S = ctx->S;
+    double *d = (double *)base;
+    int *i = (int *)(d + 4 * S);
+    return {d, d + S, d + 2 * S, d + 3 * S, i, i + S, i + 2 * S};
+}
+int ensure_host_result(rom_ctx *ctx)
+{
+    const size_t bytes = result_bytes(ctx);
+    if (ctx->h_result_cap >= bytes) return ROM_OK;
+    if (ctx->h_result) cudaFreeHost(ctx->h_result);
+    ctx->h_result = nullptr;
+    ctx->h_result_cap = 0;
+    void *p = nullptr;
+    cudaError_t e = cudaMallocHost(&p, bytes);
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();
+        return fail(ctx, ROM_ERR_OOM, "cudaMallocHost(%zu bytes): %s", bytes, cudaGetErrorString(e));
+    }
+    ctx->h_result = (unsigned char *)p;
+    ctx->h_result_cap = bytes;
     return ROM_OK;
 }
 
@@ -476,8 +515,7 @@ int build_items3(rom_ctx *ctx)
     int rc;
     if ((rc = ensure(ctx, ctx->items_dev, ctx->items.size() * sizeof(SweepItem))) ||
         (rc = ensure(ctx, ctx->cta_begin_dev, ctx->cta_begin.size() * sizeof(int))) ||
-        (rc = ensure(ctx, ctx->cta_list_dev, ctx->cta_list.size() * sizeof(int))) ||
-        (rc = ensure(ctx, ctx->err3, sizeof(int))))
+        (rc = ensure(ctx, ctx->cta_list_dev, ctx->cta_list.size() * sizeof(int))))
         return rc;
     if (ctx->n_tx > 1 &&
         (rc = ensure(ctx, ctx->xface, (size_t)total * G * ctx->K * ctx->J * sizeof(float))))
@@ -677,7 +715,7 @@ romk::SweepArgs sweep_args(const rom_ctx *ctx)
     a.leak = has_balance(ctx) ? (double *)ctx->leak.p : nullptr;
     a.dx = (float)((ctx->hi[0] - ctx->lo[0]) / ctx->I);
     a.dy = (float)((ctx->hi[1] - ctx->lo[1]) / ctx->J);
-    a.err = (int *)ctx->sweep_err.p;
+    a.err = result_view(ctx, ctx->result.p).err;
     a.wait_ns = (unsigned long long)(ctx->opt.wait_timeout_ms * 1e6);
     a.stall = ctx->opt.test_stall_waits;
     if (ctx->MOM == 0) {
@@ -721,7 +759,7 @@ romk::Sweep3Args sweep3_args(const rom_ctx *ctx)
     a.n_ty = ctx->n_ty;
     a.xface = (float *)ctx->xface.p;
     a.yface = (float *)ctx->yface.p;
-    a.err = (int *)ctx->err3.p;
+    a.err = result_view(ctx, ctx->result.p).err + 1;
     a.wait_ns = (unsigned long long)(ctx->opt.wait_timeout_ms * 1e6);
     a.stall = ctx->opt.test_stall_waits;
     return a;
@@ -788,7 +826,7 @@ int prepare_dense(rom_ctx *ctx)
         const size_t split = (size_t)ctx->Mtot * cells * 4;  // BF16 hi + lo
         const size_t ab = (size_t)ctx->S * 128 * 128 * 2;
         if ((rc = ensure(ctx, ctx->psi_split, split)) || (rc = ensure(ctx, ctx->a_hi, ab)) ||
-            (rc = ensure(ctx, ctx->a_lo, ab)) || (rc = ensure(ctx, ctx->tc_err, sizeof(int))))
+            (rc = ensure(ctx, ctx->a_lo, ab)))
             return rc;
         const void *ptrs[3] = {ctx->a_hi.p, ctx->a_lo.p, ctx->psi_split.p};
         if (memcmp(ptrs, ctx->tc_map_ptrs, sizeof ptrs) != 0 || ctx->tc_map_cells != cells ||
@@ -953,7 +991,7 @@ int enqueue_iteration(rom_ctx *ctx, cudaStream_t st, bool use_cond, cudaGraphCon
             ta.q = d.q;
             ta.src = d.src;
             ta.active = d.active;
-            ta.err = (int *)ctx->tc_err.p;
+            ta.err = result_view(ctx, ctx->result.p).err + 2;
             CK(romk::launch_dense_tc(ctx->tc_maps, ta, ctx->sm_count, st));
         } else {
             CK(romk::launch_dense_source(dense_args(ctx), max_m(ctx), st));
@@ -969,9 +1007,10 @@ int enqueue_iteration(rom_ctx *ctx, cudaStream_t st, bool use_cond, cudaGraphCon
     fa.sums = (double *)ctx->sums.p;
     fa.minkey = (int *)ctx->minkey.p;
     fa.active = (int *)ctx->active.p;
-    fa.iters = (int *)ctx->iters.p;
-    fa.flags = (int *)ctx->flags.p;
-    fa.resid = (double *)ctx->resid.p;
+    const Result res = result_view(ctx, ctx->result.p);
+    fa.iters = res.iters;
+    fa.flags = res.flags;
+    fa.resid = res.resid;
     fa.diverge_window = ctx->opt.diverge_window;
     fa.dprev = (double *)ctx->dprev.p;
     fa.grow = (int *)ctx->grow.p;
@@ -980,9 +1019,9 @@ int enqueue_iteration(rom_ctx *ctx, cudaStream_t st, bool use_cond, cudaGraphCon
     fa.dA = (ctx->hi[0] - ctx->lo[0]) / ctx->I * (ctx->hi[1] - ctx->lo[1]) / ctx->J;
     fa.sdA = batch(ctx) ? (const double *)ctx->sdA_dev.p : nullptr;
     fa.ordsum = (const double *)ctx->ordsum.p;
-    fa.bal_out = (double *)ctx->bal.p;
-    fa.leak_out = (double *)ctx->leak_out.p;
-    fa.phimin_out = (double *)ctx->phimin.p;
+    fa.bal_out = res.bal;
+    fa.leak_out = res.leak_out;
+    fa.phimin_out = res.phimin;
     fa.n_active = (int *)ctx->n_active.p;
     fa.use_cond = use_cond ? 1 : 0;
     fa.cond = h;
@@ -1075,14 +1114,25 @@ int init_state(rom_ctx *ctx)
     const int MOM = ctx->MOM == 0 ? 1 : ctx->MOM;
     const long long cells = padded_cells(ctx);
     cudaStream_t st = ctx->stream;
-    if (ctx->MOM == 0 && ctx->opt.dense_precision == 1)
-        CK(cudaMemsetAsync(ctx->tc_err.p, 0, sizeof(int), st));
-    CK(cudaMemsetAsync(ctx->sweep_err.p, 0, sizeof(int), st));
+    const Result res = result_view(ctx, ctx->result.p);
+    romk::InitState is{};
+    is.active = (int *)ctx->active.p;
+    is.iters = res.iters;
+    is.flags = res.flags;
+    is.err = res.err;
+    is.resid = res.resid;
+    is.dprev = (double *)ctx->dprev.p;
+    is.grow = (int *)ctx->grow.p;
+    is.leak = (double *)ctx->leak.p;
+    is.bal = res.bal;
+    is.leak_out = res.leak_out;
+    is.phimin = res.phimin;
+    is.sums = (double *)ctx->sums.p;
+    is.minkey = (int *)ctx->minkey.p;
     if (ctx->dim == 3) {
         // diagonal storage: sigma_T (both families), the first source q of every
         // sample, sigma_S and q for the combine (family 0), cleared accumulators, phi = 0
         const romk::Skew3 sk = romk::make_skew3(ctx->J, ctx->K, ctx->NXP);
-        CK(cudaMemsetAsync(ctx->err3.p, 0, sizeof(int), st));
         CK(cudaMemsetAsync(ctx->acc3.p, 0, 2 * (size_t)ctx->S * sk.cells * sizeof(float), st));
         CK(romk::launch_skew3_scatter((const float *)ctx->sigt.p, sk, ctx->NXP, 2, 1,
                                       (float *)ctx->sig3.p, st));
@@ -1094,13 +1144,10 @@ int init_state(rom_ctx *ctx)
                                       (float *)ctx->q3.p, st));
         ctx->launches += 4;
         CK(romk::launch_init_state(ctx->S, 1, sk.cells, nullptr, (float *)ctx->phi.p, nullptr,
-                                   (int *)ctx->active.p, (int *)ctx->iters.p, (int *)ctx->flags.p,
-                                   (double *)ctx->resid.p, st));
+                                   nullptr, is, st));
     } else if (batch(ctx)) {
         CK(cudaMemsetAsync(ctx->part.p, 0, (size_t)ctx->state_floats * sizeof(float), st));
-        CK(romk::launch_init_state(ctx->S, MOM, 0, nullptr, nullptr, nullptr, (int *)ctx->active.p,
-                                   (int *)ctx->iters.p, (int *)ctx->flags.p,
-                                   (double *)ctx->resid.p, st));
+        CK(romk::launch_init_state(ctx->S, MOM, 0, nullptr, nullptr, nullptr, nullptr, is, st));
         CK(romk::launch_init_grids(ctx->S, MOM, (const romk::GridDesc *)ctx->gdesc.p,
                                    (const int *)ctx->sgrid_dev.p, (const long long *)ctx->soff_dev.p,
                                    (int)ctx->max_cells, (const float *)ctx->q.p,
@@ -1108,11 +1155,9 @@ int init_state(rom_ctx *ctx)
         ++ctx->launches;
     } else {
         // the sweep accumulates into part; the combine clears it
-        CK(cudaMemsetAsync(ctx->part.p, 0, (size_t)ctx->S * MOM * cells * sizeof(float), st));
         CK(romk::launch_init_state(ctx->S, MOM, cells, (const float *)ctx->q.p,
-                                   (float *)ctx->phi.p, (float *)ctx->src.p, (int *)ctx->active.p,
-                                   (int *)ctx->iters.p, (int *)ctx->flags.p,
-                                   (double *)ctx->resid.p, st));
+                                   (float *)ctx->phi.p, (float *)ctx->src.p, (float *)ctx->part.p,
+                                   is, st));
     }
     ++ctx->launches;
     if (ctx->MOM == 0) {  // psi^0 = 0: every ordinate's first source is q
@@ -1120,11 +1165,6 @@ int init_state(rom_ctx *ctx)
                                    (float *)ctx->src_ord.p, st));
         ++ctx->launches;
     }
-    CK(romk::launch_init_checks(ctx->S, (double *)ctx->dprev.p, (int *)ctx->grow.p,
-                                (double *)ctx->leak.p, (double *)ctx->bal.p,
-                                (double *)ctx->leak_out.p, (double *)ctx->phimin.p,
-                                (double *)ctx->sums.p, (int *)ctx->minkey.p, st));
-    ++ctx->launches;
     if (has_balance(ctx)) {
         const unsigned char *ot = (const unsigned char *)ctx->otab.p;
         CK(romk::launch_ordsum((const double *)ctx->c64.p, (const double *)ctx->s64.p,
@@ -1134,6 +1174,18 @@ int init_state(rom_ctx *ctx)
         ++ctx->launches;
     }
     return ROM_OK;
+}
+
+// Source iterations per pass of the device-side loop: the while node costs about 2.5 us a
+// pass (4 iterations a pass: 256 x 256 x 64 samples 72.8 -> 70.6 us per iteration, 32 x 32
+// 17.9 -> 15.9), and the iterations after the last sample has stopped return at once (about
+// 2 us each).  A fixed number of sweeps takes a divisor where there is one.
+int graph_unroll(const rom_ctx *ctx)
+{
+    const int k = ctx->opt.fixed_iters;
+    for (int u : {4, 3, 2})
+        if (k > 0 && k % u == 0) return u;
+    return k == 1 ? 1 : 4;
 }
 
 int build_graph(rom_ctx *ctx)
@@ -1157,7 +1209,9 @@ int build_graph(rom_ctx *ctx)
     // stream is the legacy default stream)
     CK(cudaStreamBeginCaptureToGraph(ctx->own_stream, body, nullptr, nullptr, 0,
                                      cudaStreamCaptureModeThreadLocal));
-    int rc = enqueue_iteration(ctx, ctx->own_stream, true, h);
+    int rc = ROM_OK;
+    for (int u = 0; u < graph_unroll(ctx) && !rc; ++u)
+        rc = enqueue_iteration(ctx, ctx->own_stream, true, h);
     cudaGraph_t captured = nullptr;
     cudaError_t e = cudaStreamEndCapture(ctx->own_stream, &captured);
     if (rc) return rc;
@@ -1233,17 +1287,17 @@ void rom_destroy(rom_ctx *ctx)
     DevBuf *bufs[] = {&ctx->sigt, &ctx->sigs, &ctx->q, &ctx->inflow_dev, &ctx->c64, &ctx->s64,
                       &ctx->z64, &ctx->w64, &ctx->c32, &ctx->s32, &ctx->w32, &ctx->items_dev,
                       &ctx->phi, &ctx->src, &ctx->part, &ctx->sums, &ctx->minkey,
-                      &ctx->active, &ctx->iters, &ctx->flags, &ctx->resid, &ctx->n_active,
+                      &ctx->active, &ctx->result, &ctx->n_active,
                       &ctx->avg, &ctx->sum, &ctx->tmp, &ctx->psi, &ctx->src_ord, &ctx->Amat,
                       &ctx->dtab, &ctx->z32, &ctx->cta_begin_dev, &ctx->cta_list_dev,
-                      &ctx->xface, &ctx->yface, &ctx->err3, &ctx->sig3, &ctx->src3,
+                      &ctx->xface, &ctx->yface, &ctx->sig3, &ctx->src3,
                       &ctx->acc3, &ctx->ss3, &ctx->q3, &ctx->psi_split,
-                      &ctx->a_hi, &ctx->a_lo, &ctx->tc_err, &ctx->otab, &ctx->ordsum,
-                      &ctx->dprev, &ctx->grow,
-                      &ctx->leak, &ctx->bal, &ctx->leak_out, &ctx->phimin, &ctx->sweep_err,
+                      &ctx->a_hi, &ctx->a_lo, &ctx->otab, &ctx->ordsum, &ctx->dprev, &ctx->grow,
+                      &ctx->leak,
                       &ctx->gdesc, &ctx->sgrid_dev, &ctx->soff_dev, &ctx->sdA_dev};
     for (DevBuf *b : bufs) release(*b);
     if (ctx->h_stage) cudaFreeHost(ctx->h_stage);
+    if (ctx->h_result) cudaFreeHost(ctx->h_result);
     if (ctx->ev0) cudaEventDestroy(ctx->ev0);
     if (ctx->ev1) cudaEventDestroy(ctx->ev1);
     for (cudaEvent_t e : ctx->kev) cudaEventDestroy(e);
@@ -1683,7 +1737,7 @@ int set_ordinates_seeded(rom_ctx *ctx, uint64_t seed, int first_sample, int n_sa
     a.w32 = (float *)ctx->w32.p;
     CK(romk::launch_ordgen(a, ctx->stream));
     ++ctx->launches;
-    CK(cudaStreamSynchronize(ctx->stream));  // the packed host table dies with this call
+    // (the copy from pageable memory has taken the packed table before it returned)
     ctx->ord_source = ORD_SEED;
     ctx->seed_octants = octants;
     if (layout_same) {
@@ -1842,22 +1896,15 @@ int rom_solve(rom_ctx *ctx, rom_stats *stats_out)
     void *before[] = {ctx->phi.p,  ctx->src.p,  ctx->part.p,  ctx->sums.p, ctx->minkey.p, ctx->active.p,
                       ctx->sig3.p, ctx->src3.p, ctx->acc3.p,  ctx->ss3.p,      ctx->q3.p,
                       ctx->ordsum.p, ctx->dprev.p,
-                      ctx->grow.p, ctx->leak.p, ctx->bal.p, ctx->leak_out.p, ctx->phimin.p,
-                      ctx->sweep_err.p, ctx->otab.p};
+                      ctx->grow.p, ctx->leak.p, ctx->result.p, ctx->otab.p, ctx->gdesc.p};
     if ((rc = ensure(ctx, ctx->sums, (size_t)ctx->S * romk::kNP * sizeof(double))) ||
         (rc = ensure(ctx, ctx->minkey, (size_t)ctx->S * sizeof(int))) ||
         (rc = ensure(ctx, ctx->active, ctx->S * sizeof(int))) ||
-        (rc = ensure(ctx, ctx->iters, ctx->S * sizeof(int))) ||
-        (rc = ensure(ctx, ctx->flags, ctx->S * sizeof(int))) ||
-        (rc = ensure(ctx, ctx->resid, ctx->S * sizeof(double))) ||
+        (rc = ensure(ctx, ctx->result, result_bytes(ctx))) || (rc = ensure_host_result(ctx)) ||
         (rc = ensure(ctx, ctx->dprev, ctx->S * sizeof(double))) ||
         (rc = ensure(ctx, ctx->grow, ctx->S * sizeof(int))) ||
         (rc = ensure(ctx, ctx->leak, ctx->S * sizeof(double))) ||
-        (rc = ensure(ctx, ctx->bal, ctx->S * sizeof(double))) ||
-        (rc = ensure(ctx, ctx->leak_out, ctx->S * sizeof(double))) ||
-        (rc = ensure(ctx, ctx->phimin, ctx->S * sizeof(double))) ||
         (rc = ensure(ctx, ctx->ordsum, (size_t)ctx->S * 3 * sizeof(double))) ||
-        (rc = ensure(ctx, ctx->sweep_err, sizeof(int))) ||
         (rc = ensure(ctx, ctx->n_active, sizeof(int))) ||
         (rc = ensure(ctx, ctx->avg, nI * sizeof(double))) ||
         (rc = ensure(ctx, ctx->sum, nI * sizeof(double))))
@@ -1877,8 +1924,7 @@ int rom_solve(rom_ctx *ctx, rom_stats *stats_out)
     void *after[] = {ctx->phi.p,  ctx->src.p,  ctx->part.p,  ctx->sums.p, ctx->minkey.p, ctx->active.p,
                      ctx->sig3.p, ctx->src3.p, ctx->acc3.p,  ctx->ss3.p,      ctx->q3.p,
                      ctx->ordsum.p, ctx->dprev.p,
-                     ctx->grow.p, ctx->leak.p, ctx->bal.p, ctx->leak_out.p, ctx->phimin.p,
-                     ctx->sweep_err.p, ctx->otab.p};
+                     ctx->grow.p, ctx->leak.p, ctx->result.p, ctx->otab.p, ctx->gdesc.p};
     if (memcmp(before, after, sizeof before) != 0) invalidate_graph(ctx);
 
     const long long launches0 = ctx->launches;
@@ -1953,33 +1999,17 @@ int rom_solve(rom_ctx *ctx, rom_stats *stats_out)
                                 ctx->stream));
     ++ctx->launches;
     CK(cudaEventRecord(ctx->ev1, ctx->stream));
-    ctx->h_iters.assign(ctx->S, 0);
-    ctx->h_resid.assign(ctx->S, 0.0);
-    ctx->h_bal.assign(ctx->S, 0.0);
-    ctx->h_leak.assign(ctx->S, 0.0);
-    ctx->h_phimin.assign(ctx->S, 0.0);
-    std::vector<int> flags(ctx->S, 0);
-    int err3 = 0, tc_err = 0, sweep_err = 0;
-    if (ctx->dim == 3)
-        CK(cudaMemcpyAsync(&err3, ctx->err3.p, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaMemcpyAsync(&sweep_err, ctx->sweep_err.p, sizeof(int), cudaMemcpyDeviceToHost,
-                       ctx->stream));
-    CK(cudaMemcpyAsync(ctx->h_bal.data(), ctx->bal.p, ctx->S * sizeof(double),
-                       cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaMemcpyAsync(ctx->h_leak.data(), ctx->leak_out.p, ctx->S * sizeof(double),
-                       cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaMemcpyAsync(ctx->h_phimin.data(), ctx->phimin.p, ctx->S * sizeof(double),
-                       cudaMemcpyDeviceToHost, ctx->stream));
-    if (ctx->MOM == 0 && ctx->opt.dense_precision == 1)
-        CK(cudaMemcpyAsync(&tc_err, ctx->tc_err.p, sizeof(int), cudaMemcpyDeviceToHost,
-                           ctx->stream));
-    CK(cudaMemcpyAsync(ctx->h_iters.data(), ctx->iters.p, ctx->S * sizeof(int),
-                       cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaMemcpyAsync(ctx->h_resid.data(), ctx->resid.p, ctx->S * sizeof(double),
-                       cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaMemcpyAsync(flags.data(), ctx->flags.p, ctx->S * sizeof(int), cudaMemcpyDeviceToHost,
+    CK(cudaMemcpyAsync(ctx->h_result, ctx->result.p, result_bytes(ctx), cudaMemcpyDeviceToHost,
                        ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
+    const Result res = result_view(ctx, ctx->h_result);
+    ctx->h_iters.assign(res.iters, res.iters + ctx->S);
+    ctx->h_resid.assign(res.resid, res.resid + ctx->S);
+    ctx->h_bal.assign(res.bal, res.bal + ctx->S);
+    ctx->h_leak.assign(res.leak_out, res.leak_out + ctx->S);
+    ctx->h_phimin.assign(res.phimin, res.phimin + ctx->S);
+    const int *flags = res.flags;
+    const int sweep_err = res.err[0], err3 = res.err[1], tc_err = res.err[2];
     float ms = 0.f;
     CK(cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1));
     if (err3)
@@ -2023,7 +2053,11 @@ int rom_solve(rom_ctx *ctx, rom_stats *stats_out)
     st.source_launches = source_launches;
     st.tile_g = ctx->G_used;
     st.rows_per_step = ctx->dim == 2 ? ctx->H_used : 0;
-    if (device_loop) ctx->launches += (long long)launches_per_iteration(ctx) * st.iterations_max;
+    if (device_loop) {
+        const int u = graph_unroll(ctx);
+        ctx->launches += (long long)launches_per_iteration(ctx) *
+                         ((st.iterations_max + u - 1) / u * u);
+    }
     st.kernel_launches = ctx->launches - launches0;
     if (stats_out) *stats_out = st;
     if (diverged)

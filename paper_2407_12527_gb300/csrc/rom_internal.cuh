@@ -380,14 +380,19 @@ cudaError_t launch_extract3(const float *phi, int sample, const Skew3 &sk, int I
 cudaError_t launch_skew3_scatter(const float *in, const Skew3 &sk, int NXP, int n_fam,
                                  int n_copies, float *dst, cudaStream_t st);
 cudaError_t launch_finalize(const FinalizeArgs &a, cudaStream_t st);
+// Per-sample state of a new solve: active, no sweeps, no flags, resid and dprev = +inf,
+// grow = 0, leak = 0, bal / leak_out / phimin = NaN, sums = 0, minkey = INT_MAX; err[4] = 0.
+struct InitState {
+    int *active, *iters, *flags, *err;
+    double *resid, *dprev;
+    int *grow;
+    double *leak, *bal, *leak_out, *phimin, *sums;
+    int *minkey;
+};
+// the same launch sets phi = 0, the first source (q; nullptr: kept elsewhere) and the
+// cleared accumulators part (nullptr: not here) of [S][MOM][cells] values
 cudaError_t launch_init_state(int S, int MOM, long long cells, const float *q, float *phi,
-                              float *src, int *active, int *iters, int *flags, double *resid,
-                              cudaStream_t st);
-// per-sample divergence and balance state of a new solve: dprev = +inf, grow = 0,
-// leak = 0, bal / leak_out / phimin = NaN, sums = 0, minkey = INT_MAX
-cudaError_t launch_init_checks(int S, double *dprev, int *grow, double *leak, double *bal,
-                               double *leak_out, double *phimin, double *sums, int *minkey,
-                               cudaStream_t st);
+                              float *src, float *part, const InitState &is, cudaStream_t st);
 cudaError_t launch_average(const float *phi, int S, int MOM, int I, int J, int NXP, double *avg,
                            double *sum, cudaStream_t st);
 // several grids: phi = 0 and the first source q for every sample on its own grid
