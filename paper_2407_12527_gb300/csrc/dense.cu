@@ -61,10 +61,16 @@ __global__ void __launch_bounds__(256) pmat_kernel(const PmatArgs a)
         row[lp] = (float)(a.w[o + lp] * kernel_P(a, o + lp, o + l) * scale);
 }
 
-constexpr int BM = 128, BN = 128, BK = 8;
+// Output tile BM x BN of a CTA (8 x 8 per thread, 256 threads): 128 x 128, or for samples of
+// at most 64 or 32 ordinates 64 x 256 or 32 x 512, so that the FMAs of rows past M stay few
+// (the FMAs bound it: 8 samples of 48 ordinates on 150 x 130 cells 55 us with 128 rows, of
+// which 80 idle).  Every output element adds its k in the same order in all three.
+constexpr int BK = 8;
 
+template <int BM>
 __global__ void __launch_bounds__(256) dense_source_kernel(const DenseArgs a)
 {
+    constexpr int BN = 128 * 128 / BM, TX = BN / 8, NB = BN / 128, NA = BM / 32;
     const int s = blockIdx.z;
     if (!a.active[s]) return;
     const int M = a.M[s];
@@ -79,10 +85,10 @@ __global__ void __launch_bounds__(256) dense_source_kernel(const DenseArgs a)
     __shared__ __align__(16) float As[2][BK][BM];
     __shared__ __align__(16) float Bs[2][BK][BN];
     const int t = threadIdx.x;
-    const int tx = t & 15, ty = t >> 4;
-    // loader coordinates: A tile (BM x BK) as 4 consecutive k of one row; B tile
-    // (BK x BN) as one float4 of one row
-    const int ai = t >> 1, ak = (t & 1) * 4;
+    const int tx = t % TX, ty = t / TX;
+    // loader coordinates: A tile (BM x BK) as NA consecutive k of one row; B tile
+    // (BK x BN) as NB float4 of one row
+    const int ai = t * NA / BK, ak = t * NA % BK;
     const int bk = t >> 5, bj = (t & 31) * 4;
 
     float acc[8][8];
@@ -91,23 +97,28 @@ __global__ void __launch_bounds__(256) dense_source_kernel(const DenseArgs a)
 #pragma unroll
         for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
 
-    float ra[4];
-    float4 rb;
+    float ra[NA];
+    float4 rb[NB];
     auto gload = [&](int k0) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
+        for (int e = 0; e < NA; ++e) {
             const int m = m0 + ai, k = k0 + ak + e;
             ra[e] = (m < M && k < M) ? A[(long long)m * M + k] : 0.f;
         }
         const int k = k0 + bk;
-        const long long n = n0 + bj;
-        rb = (k < M && n < cells) ? *reinterpret_cast<const float4 *>(B + (long long)k * cells + n)
-                                  : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int e = 0; e < NB; ++e) {
+            const long long n = n0 + 128 * e + bj;
+            rb[e] = (k < M && n < cells)
+                        ? *reinterpret_cast<const float4 *>(B + (long long)k * cells + n)
+                        : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
     };
     auto sstore = [&](int buf) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) As[buf][ak + e][ai] = ra[e];
-        *reinterpret_cast<float4 *>(&Bs[buf][bk][bj]) = rb;
+        for (int e = 0; e < NA; ++e) As[buf][ak + e][ai] = ra[e];
+#pragma unroll
+        for (int e = 0; e < NB; ++e) *reinterpret_cast<float4 *>(&Bs[buf][bk][128 * e + bj]) = rb[e];
     };
 
     gload(0);
@@ -120,9 +131,9 @@ __global__ void __launch_bounds__(256) dense_source_kernel(const DenseArgs a)
 #pragma unroll
         for (int kk = 0; kk < BK; ++kk) {
             const float4 a0 = *reinterpret_cast<const float4 *>(&As[buf][kk][ty * 4]);
-            const float4 a1 = *reinterpret_cast<const float4 *>(&As[buf][kk][64 + ty * 4]);
+            const float4 a1 = *reinterpret_cast<const float4 *>(&As[buf][kk][BM / 2 + ty * 4]);
             const float4 b0 = *reinterpret_cast<const float4 *>(&Bs[buf][kk][tx * 4]);
-            const float4 b1 = *reinterpret_cast<const float4 *>(&Bs[buf][kk][64 + tx * 4]);
+            const float4 b1 = *reinterpret_cast<const float4 *>(&Bs[buf][kk][BN / 2 + tx * 4]);
             const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
             const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
@@ -140,13 +151,13 @@ __global__ void __launch_bounds__(256) dense_source_kernel(const DenseArgs a)
     // epilogue: S = sigma_S * (A psi) + q
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
-        const long long n = n0 + half * 64 + tx * 4;
+        const long long n = n0 + half * (BN / 2) + tx * 4;
         if (n >= cells) continue;
         const float4 ss = *reinterpret_cast<const float4 *>(a.sigma_s + n);
         const float4 qq = *reinterpret_cast<const float4 *>(a.q + n);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            const int m = m0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + (i - 4));
+            const int m = m0 + (i < 4 ? ty * 4 + i : BM / 2 + ty * 4 + (i - 4));
             if (m >= M) continue;
             *reinterpret_cast<float4 *>(a.src + (o + m) * cells + n) =
                 make_float4(fmaf(ss.x, acc[i][half * 4 + 0], qq.x),
@@ -180,8 +191,11 @@ cudaError_t launch_pmat(const PmatArgs &a, int max_m, cudaStream_t st)
 cudaError_t launch_dense_source(const DenseArgs &a, int max_m, cudaStream_t st)
 {
     if (a.S <= 0 || max_m <= 0) return cudaSuccess;
-    const dim3 grid((unsigned)((a.cells + BN - 1) / BN), (unsigned)((max_m + BM - 1) / BM), a.S);
-    dense_source_kernel<<<grid, 256, 0, st>>>(a);
+    const int bm = max_m <= 32 ? 32 : max_m <= 64 ? 64 : 128, bn = 128 * 128 / bm;
+    const dim3 grid((unsigned)((a.cells + bn - 1) / bn), (unsigned)((max_m + bm - 1) / bm), a.S);
+    if (bm == 32) dense_source_kernel<32><<<grid, 256, 0, st>>>(a);
+    else if (bm == 64) dense_source_kernel<64><<<grid, 256, 0, st>>>(a);
+    else dense_source_kernel<128><<<grid, 256, 0, st>>>(a);
     return cudaGetLastError();
 }
 
