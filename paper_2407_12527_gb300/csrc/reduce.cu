@@ -9,8 +9,12 @@
 //           (eq. equ_random with eq. anisotropic kernel, mirror-averaged in
 //           zeta, where sum_l' w_l' (1 + g u_l'.u_l) psi_l' = phi + g (c Jx + s Jy)),
 //           and per-block FP64 partial sums of |phi^k - phi^{k-1}|^2 and |phi^k|^2
-//           (and, in the X-Y moment modes, of sigma_T phi^k and of the previous
-//           iterate's source moments, for the particle balance), and min phi.
+//           (and, in the X-Y moment modes, of sigma_T phi^k, of the previous
+//           iterate's source and of the linear kernel's new current source
+//           moments, for the particle balance), and min phi.  The linear
+//           kernel's currents are not kept: the source moments hold them
+//           (100 x 100 x 256 samples: 50 -> 32 us per iteration beside the
+//           sweep, 2 of them the iteration loop's).
 //           Summation precision: each thread sums its few cells (8 to 32) in
 //           FP32, the 32 lanes of a warp add by an FP32 tree (5 levels), and from
 //           the warp sums on everything is FP64 (across warps, blocks and in the
@@ -95,16 +99,12 @@ __global__ void __launch_bounds__(256) combine_kernel(const CombineArgs A0)
     const long long stride = 8LL * gridDim.x * blockDim.x;
     for (long long v0 = 8 * ((long long)blockIdx.x * blockDim.x + threadIdx.x); v0 < cells;
          v0 += KS * stride) {
-        float acc[KS][MOM][8], old[KS][MOM][8], ss[KS][8], qq[KS][8], st[KS][8];
+        float acc[KS][MOM][8], old[KS][8], ss[KS][8], qq[KS][8], st[KS][8];
 #pragma unroll
         for (int k = 0; k < KS; ++k) {
             const long long v = v0 + k * stride;
             if (v >= cells) continue;
-            ld8_volatile(phi + v, old[k][0]);
-            if (MOM == 3 && A.balance) {
-                ld8_volatile(phi + cells + v, old[k][MOM == 3 ? 1 : 0]);
-                ld8_volatile(phi + 2 * cells + v, old[k][MOM == 3 ? 2 : 0]);
-            }
+            ld8_volatile(phi + v, old[k]);
 #pragma unroll
             for (int m = 0; m < MOM; ++m) ld8_volatile(A.acc + base + m * cells + v, acc[k][m]);
             ldg8(A.sigma_s + v, ss[k]);
@@ -116,18 +116,11 @@ __global__ void __launch_bounds__(256) combine_kernel(const CombineArgs A0)
             const long long v = v0 + k * stride;
             if (v >= cells) continue;
             if (A.balance) {
-                // the source moments of the previous iterate (the sweep's input) and
+                // the source moment of the previous iterate (the sweep's input) and
                 // sigma_T phi of the new one, for the particle balance; padding
                 // columns hold phi = 0 and sigma_S = q = 0
 #pragma unroll
-                for (int e = 0; e < 8; ++e) b0f += fmaf(ss[k][e], old[k][0][e], qq[k][e]);
-                if (MOM == 3) {
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        b1f = fmaf(A.g * ss[k][e], old[k][MOM == 3 ? 1 : 0][e], b1f);
-                        b2f = fmaf(A.g * ss[k][e], old[k][MOM == 3 ? 2 : 0][e], b2f);
-                    }
-                }
+                for (int e = 0; e < 8; ++e) b0f += fmaf(ss[k][e], old[k][e], qq[k][e]);
                 if (!A.sigma_t)
 #pragma unroll
                     for (int e = 0; e < 8; ++e) st[k][e] = A.sigma_t_homog;
@@ -135,7 +128,7 @@ __global__ void __launch_bounds__(256) combine_kernel(const CombineArgs A0)
             // per-element squares in FP32 (a few terms per thread), norms in FP64 below
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-                const float dd = acc[k][0][e] - old[k][0][e];
+                const float dd = acc[k][0][e] - old[k][e];
                 d2f = fmaf(dd, dd, d2f);
                 n2f = fmaf(acc[k][0][e], acc[k][0][e], n2f);
                 if (A.balance) a1f = fmaf(st[k][e], acc[k][0][e], a1f);  // sigma_T phi
@@ -148,10 +141,8 @@ __global__ void __launch_bounds__(256) combine_kernel(const CombineArgs A0)
 #pragma unroll
             for (int e = 0; e < 8; ++e) zero[e] = 0.f;
 #pragma unroll
-            for (int m = 0; m < MOM; ++m) {
-                stg8(A.acc + base + m * cells + v, zero);
-                stg8(phi + m * cells + v, acc[k][m]);
-            }
+            for (int m = 0; m < MOM; ++m) stg8(A.acc + base + m * cells + v, zero);
+            stg8(phi + v, acc[k][0]);
 #pragma unroll
             for (int e = 0; e < 8; ++e) out[e] = fmaf(ss[k][e], acc[k][0][e], qq[k][e]);
             stg8(src + v, out);
@@ -159,7 +150,10 @@ __global__ void __launch_bounds__(256) combine_kernel(const CombineArgs A0)
 #pragma unroll
                 for (int m = 1; m < 3; ++m) {
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) out[e] = A.g * ss[k][e] * acc[k][m][e];
+                    for (int e = 0; e < 8; ++e) {
+                        out[e] = A.g * ss[k][e] * acc[k][m][e];
+                        (m == 1 ? b1f : b2f) += out[e];  // of the next sweep's source
+                    }
                     stg8(src + m * cells + v, out);
                 }
             }
@@ -308,7 +302,12 @@ __global__ void __launch_bounds__(256) finalize_kernel(const FinalizeArgs A)
             A.leak[s] = 0.0;
             const double *os = A.ordsum + 3LL * s;
             const double dA = A.sdA ? A.sdA[s] : A.dA;
-            const double rhs = dA * (os[0] * b0 + os[1] * b1 + os[2] * b2);
+            // (the linear kernel's current moments come with the source they belong to, one
+            // combine earlier)
+            double *bp = A.bprev + 2LL * s;
+            const double rhs = dA * (os[0] * b0 + os[1] * bp[0] + os[2] * bp[1]);
+            bp[0] = b1;
+            bp[1] = b2;
             const double rem = dA * a1;
             const double den = fabs(lk) + fabs(rem) + fabs(rhs);
             A.bal_out[s] = den > 0.0 ? fabs(lk + rem - rhs) / den : 0.0;
@@ -385,6 +384,7 @@ __global__ void init_state_kernel(int S, int MOM, long long cells, const float *
         is.dprev[t] = (double)INFINITY;
         is.grow[t] = 0;
         is.leak[t] = 0.0;
+        is.bprev[2 * t] = is.bprev[2 * t + 1] = 0.0;
         is.bal[t] = (double)NAN;
         is.leak_out[t] = (double)NAN;
         is.phimin[t] = (double)NAN;

@@ -106,7 +106,8 @@ struct rom_ctx {
     long long max_cells = 0;         // largest grid's J * NXP
     DevBuf gdesc, sgrid_dev, soff_dev, sdA_dev;
     // per-sample divergence and balance state: dprev, grow, leak (added by the sweep)
-    DevBuf dprev, grow, leak;
+    // and the current source sums of the balance (linear kernel)
+    DevBuf dprev, grow, leak, bprev;
     // What a solve reports, in one device block and its pinned host copy, so that one copy
     // brings it back: [S] resid, bal, leak_out, phimin (of the last sweep; FP64), [S] iters,
     // flags, and the error words of the X-Y sweep, the 3D sweep and the tensor-core product.
@@ -1019,6 +1020,7 @@ int enqueue_iteration(rom_ctx *ctx, cudaStream_t st, bool use_cond, cudaGraphCon
     fa.dA = (ctx->hi[0] - ctx->lo[0]) / ctx->I * (ctx->hi[1] - ctx->lo[1]) / ctx->J;
     fa.sdA = batch(ctx) ? (const double *)ctx->sdA_dev.p : nullptr;
     fa.ordsum = (const double *)ctx->ordsum.p;
+    fa.bprev = (double *)ctx->bprev.p;
     fa.bal_out = res.bal;
     fa.leak_out = res.leak_out;
     fa.phimin_out = res.phimin;
@@ -1124,6 +1126,7 @@ int init_state(rom_ctx *ctx)
     is.dprev = (double *)ctx->dprev.p;
     is.grow = (int *)ctx->grow.p;
     is.leak = (double *)ctx->leak.p;
+    is.bprev = (double *)ctx->bprev.p;
     is.bal = res.bal;
     is.leak_out = res.leak_out;
     is.phimin = res.phimin;
@@ -1293,7 +1296,7 @@ void rom_destroy(rom_ctx *ctx)
                       &ctx->xface, &ctx->yface, &ctx->sig3, &ctx->src3,
                       &ctx->acc3, &ctx->ss3, &ctx->q3, &ctx->psi_split,
                       &ctx->a_hi, &ctx->a_lo, &ctx->otab, &ctx->ordsum, &ctx->dprev, &ctx->grow,
-                      &ctx->leak,
+                      &ctx->leak, &ctx->bprev,
                       &ctx->gdesc, &ctx->sgrid_dev, &ctx->soff_dev, &ctx->sdA_dev};
     for (DevBuf *b : bufs) release(*b);
     if (ctx->h_stage) cudaFreeHost(ctx->h_stage);
@@ -1896,7 +1899,8 @@ int rom_solve(rom_ctx *ctx, rom_stats *stats_out)
     void *before[] = {ctx->phi.p,  ctx->src.p,  ctx->part.p,  ctx->sums.p, ctx->minkey.p, ctx->active.p,
                       ctx->sig3.p, ctx->src3.p, ctx->acc3.p,  ctx->ss3.p,      ctx->q3.p,
                       ctx->ordsum.p, ctx->dprev.p,
-                      ctx->grow.p, ctx->leak.p, ctx->result.p, ctx->otab.p, ctx->gdesc.p};
+                      ctx->grow.p, ctx->leak.p, ctx->result.p, ctx->otab.p, ctx->gdesc.p,
+                      ctx->bprev.p};
     if ((rc = ensure(ctx, ctx->sums, (size_t)ctx->S * romk::kNP * sizeof(double))) ||
         (rc = ensure(ctx, ctx->minkey, (size_t)ctx->S * sizeof(int))) ||
         (rc = ensure(ctx, ctx->active, ctx->S * sizeof(int))) ||
@@ -1904,6 +1908,7 @@ int rom_solve(rom_ctx *ctx, rom_stats *stats_out)
         (rc = ensure(ctx, ctx->dprev, ctx->S * sizeof(double))) ||
         (rc = ensure(ctx, ctx->grow, ctx->S * sizeof(int))) ||
         (rc = ensure(ctx, ctx->leak, ctx->S * sizeof(double))) ||
+        (rc = ensure(ctx, ctx->bprev, 2 * ctx->S * sizeof(double))) ||
         (rc = ensure(ctx, ctx->ordsum, (size_t)ctx->S * 3 * sizeof(double))) ||
         (rc = ensure(ctx, ctx->n_active, sizeof(int))) ||
         (rc = ensure(ctx, ctx->avg, nI * sizeof(double))) ||
@@ -1924,7 +1929,8 @@ int rom_solve(rom_ctx *ctx, rom_stats *stats_out)
     void *after[] = {ctx->phi.p,  ctx->src.p,  ctx->part.p,  ctx->sums.p, ctx->minkey.p, ctx->active.p,
                      ctx->sig3.p, ctx->src3.p, ctx->acc3.p,  ctx->ss3.p,      ctx->q3.p,
                      ctx->ordsum.p, ctx->dprev.p,
-                     ctx->grow.p, ctx->leak.p, ctx->result.p, ctx->otab.p, ctx->gdesc.p};
+                     ctx->grow.p, ctx->leak.p, ctx->result.p, ctx->otab.p, ctx->gdesc.p,
+                      ctx->bprev.p};
     if (memcmp(before, after, sizeof before) != 0) invalidate_graph(ctx);
 
     const long long launches0 = ctx->launches;

@@ -27,8 +27,8 @@ constexpr int kMaxCtaItems3 = 256;  // 3D: work items per CTA list
 
 // Per-sample sums the combine blocks add (FP64 atomics) and the finalize reads
 // and clears: squared change and squared norm of phi (residual), sum of
-// sigma_T phi, sums of the three source moments of the previous iterate
-// (balance); beside them the smallest phi of the sweep as an ordered-int key.
+// sigma_T phi, sum of the previous iterate's source moment, sums of the new current
+// source moments (balance); beside them the smallest phi of the sweep as an ordered-int key.
 constexpr int kNP = 6;
 __device__ __forceinline__ int float_order_key(float f)
 {
@@ -195,6 +195,7 @@ struct FinalizeArgs {
     double dA;
     const double *sdA;          // [S] cell area per sample (several grids), else nullptr
     const double *ordsum;
+    double *bprev;              // [S][2] sums of the current source moments of the last combine
     double *bal_out, *leak_out, *phimin_out;  // [S] values of each sample's last sweep
     int *n_active;
     int use_cond;
@@ -386,7 +387,7 @@ struct InitState {
     int *active, *iters, *flags, *err;
     double *resid, *dprev;
     int *grow;
-    double *leak, *bal, *leak_out, *phimin, *sums;
+    double *leak, *bprev, *bal, *leak_out, *phimin, *sums;
     int *minkey;
 };
 // the same launch sets phi = 0, the first source (q; nullptr: kept elsewhere) and the
