@@ -42,6 +42,15 @@
 // tile hands its downstream x- and y-edges to the next tile through per-item
 // face buffers.  Every mbarrier wait is bounded in time (globaltimer): on
 // timeout the kernel raises an error flag and returns.
+//
+// What bounds it: instruction issue and latency with two warps per scheduler (about 26
+// instructions per cell and ordinate pair, of which 15 are the cell's; the loads and
+// reductions together take 13% of the time, measured without them).  128^3, 16 samples of
+// 48 ordinates: 1.69 ms per sweep, 9.5e11 updates/s (2.10 ms with the conditions on incoming
+// edges in the step, 32 arrivals per barrier phase and a packed denominator).  Measured
+// slower: 4-column strips with 16 warps per SM (3.0 ms: the per-step overhead doubles),
+// edges kept scaled by a, b, e (1.73 ms), a step without per-lane checks for the steady
+// state (1.75 ms: more code).
 #include "rom_internal.cuh"
 
 namespace romk {
@@ -78,6 +87,8 @@ __device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b)
 __device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float vsadd(float s, float a) { return s + a; }
+__device__ __forceinline__ float2 vsadd(float s, float2 a) { return make_float2(s + a.x, s + a.y); }
 __device__ __forceinline__ float vneg(float a) { return -a; }
 __device__ __forceinline__ float2 vneg(float2 a) { return make_float2(-a.x, -a.y); }
 template <class T>
@@ -195,7 +206,7 @@ __device__ __forceinline__ void block_diag(
                 continue;
             }
             const T num = vfma(a, x[h], vfma(b, y[r], vfma(e, z[h][r], vsplat<T>(pS[h][r]))));
-            const T pc = vmul(num, vrcp(vadd(vsplat<T>(pT[h][r]), abe)));
+            const T pc = vmul(num, vrcp(vsadd(pT[h][r], abe)));
             if (SCHEME == 0) {
                 const T two = vsplat<T>(2.f);
                 x[h] = vfma(two, pc, vneg(x[h]));
@@ -243,6 +254,10 @@ __device__ __forceinline__ void sweep3_body(const Sweep3Args &A, Smem3 &sm, int 
     const bool up_x = A.tile_x > 0, down_x = A.tile_x + 1 < A.n_tx;
     const bool up_y = A.tile_y > 0, down_y = A.tile_y + 1 < A.n_ty;
     const int I = A.I, J = A.J, K = A.K, NXP = A.NXP;
+    // whether edges come in from a face or another tile; without, they are zero, and the
+    // loads and their conditions stay out of the step (their instructions were a quarter of
+    // the sweep's time)
+    const bool edge_y = up_y || A.inflow != nullptr, edge_x = up_x || A.inflow != nullptr;
     const long long plane = A.sk.DS;  // one z-plane further: one diagonal further
     const int fam = yneg == zneg ? 0 : 1;
     const float *const sig_f = A.sigma_t + (long long)fam * A.sk.cells;
@@ -339,7 +354,10 @@ __device__ __forceinline__ void sweep3_body(const Sweep3Args &A, Smem3 &sm, int 
         const int k = zneg ? K - 1 - kl : kl;
         // incoming x-edges of the lane's rows
         if (first_x) {
-            if (act) {
+            if (!edge_x) {
+#pragma unroll
+                for (int h = 0; h < kH3; ++h) xin[h] = vsplat<T>(0.f);
+            } else if (act) {
 #pragma unroll
                 for (int h = 0; h < kH3; ++h)
 #pragma unroll
@@ -373,10 +391,15 @@ __device__ __forceinline__ void sweep3_body(const Sweep3Args &A, Smem3 &sm, int 
                 vset(xin[2], 0, v1.x); vset(xin[2], 1, v1.y);
                 vset(xin[3], 0, v1.z); vset(xin[3], 1, v1.w);
             }
-            mbar_arrive(&sm.empty[w - 1][slot]);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sm.empty[w - 1][slot]);
         }
         // incoming y-edges of the first row block (the others arrive by shuffle)
-        if (lane == 0 && act) {
+        if (!edge_y) {
+#pragma unroll
+            for (int r = 0; r < kCols; ++r)
+                if (lane == 0) y[r] = vsplat<T>(0.f);
+        } else if (lane == 0 && act) {
 #pragma unroll
             for (int r = 0; r < kCols; ++r)
 #pragma unroll
@@ -439,7 +462,8 @@ __device__ __forceinline__ void sweep3_body(const Sweep3Args &A, Smem3 &sm, int 
                 sm.ring[w][slot][lane][0] = make_float4(xo[0].x, xo[0].y, xo[1].x, xo[1].y);
                 sm.ring[w][slot][lane][1] = make_float4(xo[2].x, xo[2].y, xo[3].x, xo[3].y);
             }
-            mbar_arrive(&sm.full[w][slot]);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sm.full[w][slot]);
         }
         // outgoing y-edges: the last row block of the tile to the next tile
         if (down_y && act && lane == NB - 1) {
@@ -496,8 +520,8 @@ __global__ void __launch_bounds__(32 * kStrips, 1) sweep3d_kernel(const Sweep3Ar
         }
         if (lane == 0) sm.n_list = n;
         for (int i = lane; i < kStrips * kSlots; i += 32) {
-            mbar_init(&sm.full[i / kSlots][i % kSlots], 32);
-            mbar_init(&sm.empty[i / kSlots][i % kSlots], 32);
+            mbar_init(&sm.full[i / kSlots][i % kSlots], 1);  // (the warp's lane 0 arrives)
+            mbar_init(&sm.empty[i / kSlots][i % kSlots], 1);
         }
         if (lane == 0) mbar_init(&sm.never, 1);
     }
