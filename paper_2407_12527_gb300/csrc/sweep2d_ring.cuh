@@ -35,7 +35,9 @@
 // The uniform case takes five packed FP32x2 operations per cell and ordinate pair and its
 // upwind chain is one FMA per cell.  The DD closure keeps -P after even steps (and the
 // varying case -X at odd cells), so that every update is one FMA without a negated operand:
-// P' = c - P or -P' = P - c.
+// P' = c - P or -P' = P - c.  (Negated operands cost the packed instructions nothing; the
+// plain form measured 4% slower on the checkerboard with four ordinates per item, 7% faster
+// on three mixed grids with two, the same elsewhere.)
 //
 // What bounds it.  A warp issues 115-125 instructions per step of 512 updates at 2.5-3
 // cycles each with the one or two warps per scheduler of most solves (fixed-latency
