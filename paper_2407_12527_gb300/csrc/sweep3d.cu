@@ -46,7 +46,7 @@
 // What bounds it: instruction issue and latency with two warps per scheduler (about 26
 // instructions per cell and ordinate pair, of which 15 are the cell's; the loads and
 // reductions together take 13% of the time, measured without them).  128^3, 16 samples of
-// 48 ordinates: 1.69 ms per sweep, 9.5e11 updates/s (2.10 ms with the conditions on incoming
+// 48 ordinates: 1.67 ms per sweep, 9.7e11 updates/s (2.10 ms with the conditions on incoming
 // edges in the step, 32 arrivals per barrier phase and a packed denominator).  Measured
 // slower: 4-column strips with 16 warps per SM (3.0 ms: the per-step overhead doubles),
 // edges kept scaled by a, b, e (1.73 ms), a step without per-lane checks for the steady
@@ -114,6 +114,11 @@ __device__ __forceinline__ float rcp_approx(float x)
 }
 __device__ __forceinline__ float vrcp(float a) { return rcp_approx(a); }
 __device__ __forceinline__ float2 vrcp(float2 a) { return make_float2(rcp_approx(a.x), rcp_approx(a.y)); }
+__device__ __forceinline__ float vsel(bool c, float a, float b) { return c ? a : b; }
+__device__ __forceinline__ float2 vsel(bool c, float2 a, float2 b)
+{
+    return make_float2(c ? a.x : b.x, c ? a.y : b.y);
+}
 // sum over the ordinates of w_g psi_g
 __device__ __forceinline__ float wsum(float w, float p) { return w * p; }
 __device__ __forceinline__ float wsum(float2 w, float2 p) { return fmaf(w.y, p.y, w.x * p.x); }
@@ -178,8 +183,15 @@ __device__ __forceinline__ void red8(float *p, const float (&v)[kCols])
 // cells are taken by anti-diagonals of the block (cell (h, r) at diagonal h + r,
 // r counted from the x inflow side), so the up to four cells of a diagonal are
 // independent and their dependent FMA chains overlap.  A row's flux goes out
-// (one vector reduction per 4 cells) as soon as the row is done, and its source
-// and sigma_T registers are reloaded with the row of the next step.
+// (one vector reduction per 4 cells) as soon as the row is done, after its source
+// and sigma_T registers are reloaded with the row of the next step (loads before the
+// reductions: 127 against 130 us on 45 x 38 x 52, the same on 128^3).
+//
+// CHECK: some lanes' rows, or columns of the strip, lie outside the grid.  Such cells are
+// computed like the others (their source stays 0 and sigma_T 1) and their results dropped
+// by selects: the y-edges pass a row outside, the x-edges a column outside, no flux goes
+// out.  (With a branch per cell 45 x 38 x 52, 8 samples of 32, measured
+// 176 us per sweep instead of 130.)
 template <int G, int SCHEME, bool XNEG, bool CHECK>
 __device__ __forceinline__ void block_diag(
     const typename V3<G>::T a, const typename V3<G>::T b, const typename V3<G>::T e,
@@ -201,33 +213,30 @@ __device__ __forceinline__ void block_diag(
             const int rr = d - h;
             if (rr < 0 || rr >= kCols) continue;
             const int r = XNEG ? kCols - 1 - rr : rr;
-            if (CHECK && !(rok[h] && cok[r])) {
-                out[h][r] = 0.f;
-                continue;
-            }
             const T num = vfma(a, x[h], vfma(b, y[r], vfma(e, z[h][r], vsplat<T>(pS[h][r]))));
             const T pc = vmul(num, vrcp(vsadd(pT[h][r], abe)));
+            T xn = pc, yn = pc;
             if (SCHEME == 0) {
                 const T two = vsplat<T>(2.f);
-                x[h] = vfma(two, pc, vneg(x[h]));
-                y[r] = vfma(two, pc, vneg(y[r]));
+                xn = vfma(two, pc, vneg(x[h]));
+                yn = vfma(two, pc, vneg(y[r]));
                 z[h][r] = vfma(two, pc, vneg(z[h][r]));
             } else {
-                x[h] = pc;
-                y[r] = pc;
                 z[h][r] = pc;
             }
-            out[h][r] = wsum(wg, pc);
+            x[h] = vsel(!CHECK || cok[r], xn, x[h]);
+            y[r] = vsel(!CHECK || rok[h], yn, y[r]);
+            out[h][r] = !CHECK || cok[r] ? wsum(wg, pc) : 0.f;
         }
         const int hf = d - (kCols - 1);  // the row finished at this diagonal
         if (hf >= 0 && hf < kH3) {
             xo[hf] = x[hf];
             if (!CHECK || rok[hf]) {
-                red8(phi_k + rowpart[hf], out[hf]);
                 if (act2) {
                     ld8_volatile(sp2 + rowpart[hf], pS[hf]);
                     ld8_volatile(tp2 + rowpart[hf], pT[hf]);
                 }
+                red8(phi_k + rowpart[hf], out[hf]);
             }
         }
     }
@@ -294,7 +303,11 @@ __device__ __forceinline__ void sweep3_body(const Sweep3Args &A, Smem3 &sm, int 
     for (int h = 0; h < kH3; ++h) {
         xin[h] = vsplat<T>(0.f);
 #pragma unroll
-        for (int r = 0; r < kCols; ++r) z[h][r] = vsplat<T>(0.f);
+        for (int r = 0; r < kCols; ++r) {
+            z[h][r] = vsplat<T>(0.f);
+            pS[h][r] = 0.f;
+            pT[h][r] = 1.f;
+        }
     }
 #pragma unroll
     for (int r = 0; r < kCols; ++r) y[r] = vsplat<T>(0.f);
