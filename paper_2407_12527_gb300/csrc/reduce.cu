@@ -267,67 +267,79 @@ __global__ void skew3_scatter_kernel(const float *in, Skew3 g, int NXP, int n_fa
     }
 }
 
-__global__ void __launch_bounds__(256) finalize_kernel(const FinalizeArgs A)
+// One warp per 32 samples, each on an SM of its own: the FP64 square root and divisions of 256
+// samples kept one SM's two FP64 lanes busy for about 3 us, and one sample's chain of loads
+// waited on each other.  Per iteration, one block of 256 threads against this form: 16.4 ->
+// 15.1 us on 32 x 32 (one sample), 45.7 -> 44.1 on 256 x 256 (one sample), 84.9 -> 83.4 on
+// 100 x 100 x 256 samples (linear kernel).  In the combine's last block instead, behind a
+// fence and an arrival count, it cost 2 us more than the launch it saved.
+// All loads come first (a sample that is not active loads its state too), the comparison of
+// successive changes is one of squares.  Several warps count the samples that go on in one
+// word, arrivals in its upper half; the last one resets it.
+__global__ void __launch_bounds__(32) finalize_kernel(const FinalizeArgs A)
 {
-    int cnt = 0;
-    for (int s = threadIdx.x; s < A.S; s += blockDim.x) {
-        if (!A.active[s]) continue;
-        // the sums the combine blocks added, cleared for the next sweep
-        double *sm = A.sums + (long long)s * kNP;
+    const int s = blockIdx.x * 32 + threadIdx.x;
+    bool go = false;
+    if (s < A.S) {
+        double *sm = A.sums + (long long)s * kNP, *bp = A.bprev + 2LL * s;
+        const int act = A.active[s], mk = A.minkey[s], it = A.iters[s] + 1, grow = A.grow[s];
         const double d2 = sm[0], n2 = sm[1], a1 = sm[2], b0 = sm[3], b1 = sm[4], b2 = sm[5];
-#pragma unroll
-        for (int k = 0; k < kNP; ++k) sm[k] = 0.0;
-        const int mk = A.minkey[s];
-        A.minkey[s] = 0x7FFFFFFF;
-        const double mn = mk == 0x7FFFFFFF ? (double)NAN : (double)float_from_order_key(mk);
-        const double r = n2 > 0.0 ? sqrt(d2 / n2) : (d2 == 0.0 ? 0.0 : (double)INFINITY);
-        const int it = A.iters[s] + 1;
-        A.iters[s] = it;
-        A.resid[s] = r;
-        const bool bad = !isfinite(r);
-        // divergence: the change ||phi^k - phi^{k-1}|| itself grows sweep after
-        // sweep (for a contracting iteration it shrinks by the spectral radius)
-        const double dn = sqrt(d2);
-        const int gr = (dn > A.dprev[s] && !(r < A.tol)) ? A.grow[s] + 1 : 0;
-        A.grow[s] = gr;
-        A.dprev[s] = dn;
-        const bool growing = A.diverge_window > 0 && gr >= A.diverge_window;
-        if (bad) A.flags[s] |= 1;
-        if (growing) A.flags[s] |= 2;
-        A.phimin_out[s] = mn;
+        const double d2prev = A.dprev[s];
+        double lk = 0.0, o0 = 0.0, o1 = 0.0, o2 = 0.0, c0 = 0.0, c1 = 0.0, dA = A.dA;
         if (A.balance) {
-            // leakage + sum sigma_T phi^k dA = sum_l w_l sum S_l^{k-1} dA, exact for
-            // the cell equations of the sweep up to its rounding
-            const double lk = A.leak[s];
-            A.leak[s] = 0.0;
             const double *os = A.ordsum + 3LL * s;
-            const double dA = A.sdA ? A.sdA[s] : A.dA;
-            // (the linear kernel's current moments come with the source they belong to, one
-            // combine earlier)
-            double *bp = A.bprev + 2LL * s;
-            const double rhs = dA * (os[0] * b0 + os[1] * bp[0] + os[2] * bp[1]);
-            bp[0] = b1;
-            bp[1] = b2;
-            const double rem = dA * a1;
-            const double den = fabs(lk) + fabs(rem) + fabs(rhs);
-            A.bal_out[s] = den > 0.0 ? fabs(lk + rem - rhs) / den : 0.0;
-            A.leak_out[s] = lk;
+            lk = A.leak[s];
+            o0 = os[0], o1 = os[1], o2 = os[2];
+            c0 = bp[0], c1 = bp[1];
+            if (A.sdA) dA = A.sdA[s];
         }
-        bool stop;
-        if (A.fixed_iters > 0) stop = it >= A.fixed_iters;
-        else stop = (r < A.tol) || it >= A.max_iter || bad || growing;
-        if (stop) A.active[s] = 0;
-        else ++cnt;
-    }
-    __shared__ int red[32];
+        if (act) {
+            // the sums the combine blocks added, cleared for the next sweep
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = cnt;
-    __syncthreads();
+            for (int k = 0; k < kNP; ++k) sm[k] = 0.0;
+            A.minkey[s] = 0x7FFFFFFF;
+            const double mn = mk == 0x7FFFFFFF ? (double)NAN : (double)float_from_order_key(mk);
+            const double r = n2 > 0.0 ? sqrt(d2 / n2) : (d2 == 0.0 ? 0.0 : (double)INFINITY);
+            A.iters[s] = it;
+            A.resid[s] = r;
+            const bool bad = !isfinite(r);
+            // divergence: the change ||phi^k - phi^{k-1}|| itself grows sweep after
+            // sweep (for a contracting iteration it shrinks by the spectral radius)
+            const int gr = (d2 > d2prev && !(r < A.tol)) ? grow + 1 : 0;
+            A.grow[s] = gr;
+            A.dprev[s] = d2;
+            const bool growing = A.diverge_window > 0 && gr >= A.diverge_window;
+            if (bad || growing) A.flags[s] |= (bad ? 1 : 0) | (growing ? 2 : 0);
+            A.phimin_out[s] = mn;
+            if (A.balance) {
+                // leakage + sum sigma_T phi^k dA = sum_l w_l sum S_l^{k-1} dA, exact for
+                // the cell equations of the sweep up to its rounding
+                A.leak[s] = 0.0;
+                // (the linear kernel's current moments come with the source they belong to,
+                // one combine earlier)
+                const double rhs = dA * (o0 * b0 + o1 * c0 + o2 * c1);
+                bp[0] = b1;
+                bp[1] = b2;
+                const double rem = dA * a1;
+                const double den = fabs(lk) + fabs(rem) + fabs(rhs);
+                A.bal_out[s] = den > 0.0 ? fabs(lk + rem - rhs) / den : 0.0;
+                A.leak_out[s] = lk;
+            }
+            if (A.fixed_iters > 0) go = it < A.fixed_iters;
+            else go = !((r < A.tol) || it >= A.max_iter || bad || growing);
+            if (!go) A.active[s] = 0;
+        }
+    }
+    const unsigned cnt = __popc(__ballot_sync(0xffffffffu, go));
     if (threadIdx.x == 0) {
-        int tot = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += red[w];
-        *A.n_active = tot;
+        unsigned tot = cnt;
+        if (gridDim.x > 1) {
+            const unsigned long long old = atomicAdd(A.going, (1ull << 32) | cnt);
+            if ((unsigned)(old >> 32) != gridDim.x - 1) return;
+            tot += (unsigned)old;
+            *A.going = 0;
+        }
+        *A.n_active = (int)tot;
         if (A.use_cond) cudaGraphSetConditional(A.cond, tot > 0 ? 1u : 0u);
     }
 }
@@ -376,6 +388,7 @@ __global__ void init_state_kernel(int S, int MOM, long long cells, const float *
     if (blockIdx.y > 0) return;
     const int t0 = blockIdx.x * blockDim.x + threadIdx.x;
     if (t0 < 4) is.err[t0] = 0;
+    if (t0 == 0) *is.going = 0;
     for (long long t = t0; t < S; t += (long long)gridDim.x * blockDim.x) {
         is.active[t] = 1;
         is.iters[t] = 0;
@@ -533,7 +546,7 @@ cudaError_t launch_skew3_scatter(const float *in, const Skew3 &sk, int NXP, int 
 
 cudaError_t launch_finalize(const FinalizeArgs &a, cudaStream_t st)
 {
-    finalize_kernel<<<1, 256, 0, st>>>(a);
+    finalize_kernel<<<(a.S + 31) / 32, 32, 0, st>>>(a);
     return cudaGetLastError();
 }
 

@@ -1005,6 +1005,7 @@ int enqueue_iteration(rom_ctx *ctx, cudaStream_t st, bool use_cond, cudaGraphCon
     fa.leak_out = res.leak_out;
     fa.phimin_out = res.phimin;
     fa.n_active = (int *)ctx->n_active.p;
+    fa.going = (unsigned long long *)ctx->n_active.p + 1;
     fa.use_cond = use_cond ? 1 : 0;
     fa.cond = h;
     CK(romk::launch_finalize(fa, st));
@@ -1134,6 +1135,7 @@ int init_state(rom_ctx *ctx)
     is.phimin = res.phimin;
     is.sums = (double *)ctx->sums.p;
     is.minkey = (int *)ctx->minkey.p;
+    is.going = (unsigned long long *)ctx->n_active.p + 1;
     if (ctx->dim == 3) {
         // diagonal storage: sigma_T (both families), the first source q of every
         // sample, sigma_S and q for the combine (family 0), cleared accumulators, phi = 0
@@ -1912,7 +1914,7 @@ int rom_solve(rom_ctx *ctx, rom_stats *stats_out)
         (rc = ensure(ctx, ctx->leak, ctx->S * sizeof(double))) ||
         (rc = ensure(ctx, ctx->bprev, 2 * ctx->S * sizeof(double))) ||
         (rc = ensure(ctx, ctx->ordsum, (size_t)ctx->S * 3 * sizeof(double))) ||
-        (rc = ensure(ctx, ctx->n_active, sizeof(int))) ||
+        (rc = ensure(ctx, ctx->n_active, 2 * sizeof(unsigned long long))) ||
         (rc = ensure(ctx, ctx->avg, nI * sizeof(double))) ||
         (rc = ensure(ctx, ctx->sum, nI * sizeof(double))))
         return rc;

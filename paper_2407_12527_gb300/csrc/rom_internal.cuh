@@ -185,7 +185,7 @@ struct FinalizeArgs {
     int *minkey;                // [S] read and reset
     int *active, *iters, *flags;
     double *resid;
-    double *dprev;              // [S] ||phi^k - phi^{k-1}||_2 of the previous sweep
+    double *dprev;              // [S] squared ||phi^k - phi^{k-1}||_2 of the previous sweep
     int *grow;                  // [S] consecutive sweeps whose change grew
     // particle balance of the sweep (balance != 0): the net leakage the sweep
     // added per sample (read and cleared), the cell area and per-sample sums
@@ -198,6 +198,7 @@ struct FinalizeArgs {
     double *bprev;              // [S][2] sums of the current source moments of the last combine
     double *bal_out, *leak_out, *phimin_out;  // [S] values of each sample's last sweep
     int *n_active;
+    unsigned long long *going;  // (blocks done, samples going on), 0 between launches
     int use_cond;
     cudaGraphConditionalHandle cond;
 };
@@ -382,13 +383,15 @@ cudaError_t launch_skew3_scatter(const float *in, const Skew3 &sk, int NXP, int 
                                  int n_copies, float *dst, cudaStream_t st);
 cudaError_t launch_finalize(const FinalizeArgs &a, cudaStream_t st);
 // Per-sample state of a new solve: active, no sweeps, no flags, resid and dprev = +inf,
-// grow = 0, leak = 0, bal / leak_out / phimin = NaN, sums = 0, minkey = INT_MAX; err[4] = 0.
+// grow = 0, leak = 0, bal / leak_out / phimin = NaN, sums = 0, minkey = INT_MAX; err[4] = 0,
+// going = 0.
 struct InitState {
     int *active, *iters, *flags, *err;
     double *resid, *dprev;
     int *grow;
     double *leak, *bprev, *bal, *leak_out, *phimin, *sums;
     int *minkey;
+    unsigned long long *going;
 };
 // the same launch sets phi = 0, the first source (q; nullptr: kept elsewhere) and the
 // cleared accumulators part (nullptr: not here) of [S][MOM][cells] values
