@@ -139,6 +139,9 @@ struct rom_ctx {
     int MOM = 1;  // 1 isotropic moments, 3 linear moments, 0 dense operator
     int chunks = 1;
     DevBuf phi, src, part, sums, minkey, active, n_active, avg, sum, tmp;
+    // host table of the last seeded ordinate set, and whether its upload may be in flight
+    std::vector<unsigned char> seed_table;
+    bool seed_upload = false;
     bool solved = false;
     std::vector<int> h_iters;
     std::vector<double> h_resid;
@@ -1674,6 +1677,11 @@ int set_ordinates_seeded(rom_ctx *ctx, uint64_t seed, int first_sample, int n_sa
     if ((long long)first_sample + n_samples > (1LL << 31))
         return fail(ctx, ROM_ERR_INVALID_ARG, "sample index out of range");
     CK(cudaSetDevice(ctx->device));
+    // a captured upload would read the host table again at every replay
+    cudaStreamCaptureStatus capturing;
+    CK(cudaStreamIsCapturing(ctx->stream, &capturing));
+    if (capturing != cudaStreamCaptureStatusNone)
+        return fail(ctx, ROM_ERR_CUDA, "ordinate sets cannot be drawn while the stream is captured");
     const bool same_layout =
         ctx->ord_source == ORD_SEED && ctx->S == n_samples && ctx->seed_octants == octants;
     const int per_cell = octants ? 8 : 4;
@@ -1705,11 +1713,15 @@ int set_ordinates_seeded(rom_ctx *ctx, uint64_t seed, int first_sample, int n_sa
         (rc = ensure(ctx, ctx->c32, b4)) || (rc = ensure(ctx, ctx->s32, b4)) ||
         (rc = ensure(ctx, ctx->z32, b4)) || (rc = ensure(ctx, ctx->w32, b4)))
         return rc;
-    // small per-sample tables packed into one device buffer
+    // small per-sample tables packed into one device buffer; their host copy stays with the
+    // context, so that the call need not wait for the upload
     const size_t tb = (size_t)n_samples * (2 * sizeof(int) + sizeof(long long)) +
                       (size_t)(n_samples + 1) * sizeof(int) + 64;
     if ((rc = ensure(ctx, ctx->tmp, tb))) return rc;
-    std::vector<unsigned char> packed(tb, 0);
+    if (ctx->seed_upload) CK(cudaStreamSynchronize(ctx->stream));  // the last one's table
+    ctx->seed_upload = false;
+    std::vector<unsigned char> &packed = ctx->seed_table;
+    packed.assign(tb, 0);
     size_t p = 0;
     const size_t o_off = p;
     memcpy(packed.data() + p, off.data(), n_samples * sizeof(long long));
@@ -1722,6 +1734,7 @@ int set_ordinates_seeded(rom_ctx *ctx, uint64_t seed, int first_sample, int n_sa
     p += n_samples * sizeof(int);
     const size_t o_fc = p;
     memcpy(packed.data() + p, first_cell.data(), (n_samples + 1) * sizeof(int));
+    ctx->seed_upload = true;
     CK(cudaMemcpyAsync(ctx->tmp.p, packed.data(), tb, cudaMemcpyHostToDevice, ctx->stream));
     romk::OrdGenArgs a{};
     unsigned char *base = (unsigned char *)ctx->tmp.p;
@@ -1744,7 +1757,6 @@ int set_ordinates_seeded(rom_ctx *ctx, uint64_t seed, int first_sample, int n_sa
     a.w32 = (float *)ctx->w32.p;
     CK(romk::launch_ordgen(a, ctx->stream));
     ++ctx->launches;
-    // (the copy from pageable memory has taken the packed table before it returned)
     ctx->ord_source = ORD_SEED;
     ctx->seed_octants = octants;
     if (layout_same) {
@@ -2013,6 +2025,7 @@ int rom_solve(rom_ctx *ctx, rom_stats *stats_out)
     CK(cudaMemcpyAsync(ctx->h_result, ctx->result.p, result_bytes(ctx), cudaMemcpyDeviceToHost,
                        ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
+    ctx->seed_upload = false;
     const Result res = result_view(ctx, ctx->h_result);
     ctx->h_iters.assign(res.iters, res.iters + ctx->S);
     ctx->h_resid.assign(res.resid, res.resid + ctx->S);
