@@ -38,6 +38,8 @@ METRIC = "cell-ordinate updates/s (ROM source iteration, 1 GB300)"
 UNIT = "updates/s"
 FLOP_PER_UPDATE = 11  # diamond difference, homogeneous sigma_T: 5 FMA + 1 MUL
 FLOP_PER_UPDATE_HET = 13  # heterogeneous sigma_T: + 1 add + 1 reciprocal per cell-ordinate
+FLOP_PER_UPDATE_RING = 8       # one-row sweep: 2 ADD + 3 FMA in scaled edge fluxes
+FLOP_PER_UPDATE_RING_HET = 11  # varying sigma_T: 3 ADD + reciprocal + MUL + 3 FMA
 FLOP_PER_UPDATE_3D = 17   # 3D, heterogeneous: 3 FMA + add + reciprocal + MUL, 3 FMA outflows, 1 FMA phi
 TOL = 1e-6
 DENSE_SWEEP_BYTES_PER_UPDATE = 8  # dense-mode sweep: FP32 source read + BF16 hi/lo psi written
@@ -452,6 +454,7 @@ def run_ours(args):
         src_n += s["source_launches"]
         if WL.kernel == "hg":  # 2 M^2 flops per cell and contraction, per active sample
             it, _ = ctx.iterations()
+            it = np.asarray(it) - 1  # (no contraction after a sample's last sweep)
             M = 4 * WL.nz[0] * WL.nt[0]
             src_flop += 2.0 * M * M * p.I * p.J * float(np.sum(it))
             # algorithmic HBM bytes of a contraction: psi read + sources written, 4 B each
@@ -461,7 +464,9 @@ def run_ours(args):
                     dense_precision=args.dense_precision)
     peak_tflops = 152 * 128 * 2 * 2070e6 / 1e12
     homog = float(np.min(p.sigma_t)) == float(np.max(p.sigma_t))
-    fpu = FLOP_PER_UPDATE_3D if WL.dim == 3 else (FLOP_PER_UPDATE if homog else FLOP_PER_UPDATE_HET)
+    fpu = (FLOP_PER_UPDATE_3D if WL.dim == 3 else
+           (FLOP_PER_UPDATE_RING if homog else FLOP_PER_UPDATE_RING_HET) if s["rows_per_step"] == 1
+           else FLOP_PER_UPDATE if homog else FLOP_PER_UPDATE_HET)
     hbm_peak = measured_hbm_gbs()
     tc = WL.kernel == "hg" and args.dense_precision == 1
     if WL.kernel == "hg" and src_ms > 0 and tc:
@@ -475,7 +480,7 @@ def run_ours(args):
     else:
         achieved = sweep_upd * fpu / (sweep_ms / 1e3) / 1e12
         kernel_name = ("sweep3d_kernel (K9)" if WL.dim == 3 else
-                       "sweep2d_row_kernel (K1, one row per step)" if s["rows_per_step"] == 1
+                       "sweep2d_ring_kernel (K1, one row per step)" if s["rows_per_step"] == 1
                        else "sweep2d_kernel (K1, %d rows per step)" % s["rows_per_step"])
         kernel_name, n_l, avg_us, fu = (kernel_name, sweep_n, 1e3 * sweep_ms / max(sweep_n, 1), fpu)
     # DRAM bytes of one full launch from the committed ncu captures, used only
@@ -486,8 +491,8 @@ def run_ours(args):
                                  shape="G%dH%d" % (s["tile_g"], s["rows_per_step"]))
     elif WL.name == "lognormal_cube" and s["tile_g"] == 2:
         traffic = traffic_record("sweep3d_lognormal_cube_128", "sweep3d.cu", WL.samples)
-    elif WL.name == "checkerboard" and s["tile_g"] == 4 and s["rows_per_step"] == 2:
-        traffic = traffic_record("sweep2d_checkerboard_448", "sweep2d_impl.cuh", WL.samples)
+    elif WL.name == "checkerboard" and s["tile_g"] == 4 and s["rows_per_step"] == 1:
+        traffic = traffic_record("sweep2d_checkerboard_448", "sweep2d_ring.cuh", WL.samples)
     if tc and src_ms > 0:
         roofline = {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                     "frac": achieved / hbm_peak,
@@ -509,11 +514,11 @@ def run_ours(args):
             roofline = {"bound": "hbm", "achieved": sw, "peak": hbm_peak, "unit": "GB/s",
                         "frac": sw / hbm_peak,
                         "traffic": traffic_record("sweep2d_dense_hg_disc_512",
-                                                  "sweep2d_impl.cuh", WL.samples),
+                                                  "sweep2d_ring.cuh", WL.samples),
                         "traffic_note": "DRAM read+write bytes of one launch with every sample "
                                         "active (ncu, scaled by samples); achieved counts the "
                                         "algorithmic bytes, 8 B per cell-ordinate update",
-                        "kernel": "sweep2d_kernel (K1, dense mode: per-ordinate sources in, "
+                        "kernel": "sweep2d_ring_kernel (K1, dense mode: per-ordinate sources in, "
                                   "split-BF16 psi out)",
                         "launches": sweep_n, "avg_launch_us": 1e3 * sweep_ms / max(sweep_n, 1),
                         "bytes_per_update": DENSE_SWEEP_BYTES_PER_UPDATE,
