@@ -1055,9 +1055,11 @@ int autotune_g(rom_ctx *ctx)
     for (int cand = 0; cand < 9; ++cand) {
         const int G = 1 << (cand / 3), H = 1 << (cand % 3);  // H = 1, 2, 4
         if (G > cap || (want_h != 0 && H != want_h) || (dense && H == 2)) continue;
-        // the ring-staged one-row kernel, where it runs, beats the 2- and 4-row shapes, and
-        // has no one-ordinate form
-        if (ring && (G == 1 || (want_h == 0 && H != 1)) && !(want_h > 1)) continue;
+        // where the ring-staged one-row kernel runs it has no one-ordinate form, and of the
+        // others only two rows per step come near it: with varying sigma_T and inflow (256 x
+        // 128, 300 samples of 16 124 us against 164) or the linear kernel (144 x 128 149
+        // against 204)
+        if (ring && (G == 1 || (want_h == 0 && H == 4)) && !(want_h > 1)) continue;
         ctx->opt.tile_g = G;
         if ((rc = build_items(ctx))) return rc;
         if ((rc = ensure_state(ctx))) return rc;  // phi, sources, accumulators

@@ -19,11 +19,35 @@ cudaError_t launch_sweep2d_ring_dense(const SweepArgs &a, int n_items, int C, in
 
 namespace {
 
-// Cells per lane.  8 halve the per-step overhead per cell and the number of warps; 4 are
-// faster for rows one warp covers, and where there are fewer than two items per SM to share
-// the schedulers (256 x 256, 128 items of 2 ordinates: 34.9 us per sweep against 42.8; 256
-// items of 4: 53.2 against 56.9; 1024 items of 4: 133 against 92).
-int cells_per_lane(int I, int n_items) { return I > 128 && n_items >= 2 * 152 ? 8 : 4; }
+// Cells per lane.  8 halve the per-step overhead per cell and the number of warps; 4 take
+// half the registers and rings per warp (more CTAs per SM, a smoother last wave) and round the
+// width to 128 cells instead of 256.  Microseconds per sweep, 8 against 4 cells, samples of 16:
+//   up to 256 wide: 8, unless there are too few items to share the schedulers (2 per SM, of
+//     four ordinates 3, with inflow 4: 256 x 256, 1200 items of two 89 against 126, 128 of two
+//     43 against 35; 600 of four 64 against 80; three grids up to 200 wide, 384 of four 108
+//     against 74; 211 x 173 with inflow, varying sigma_T, 384 of two 87 against 73);
+//   257 .. 384 (more generally where 256-cell warps round up further): 4 (320 x 256, varying
+//     sigma_T, 600 of four 261 against 145), but for uniform sigma_T with two ordinates (147
+//     against 176);
+//   above: 8 (512 x 256 uniform 184 against 250), but for varying sigma_T with four ordinates,
+//     whose 220 registers and 64 KB of rings want many long items (448 x 64, 2000 items 395
+//     against 319; 448 x 448, 2048 of uneven samples 945 against 1000);
+//   inflow with varying sigma_T and four ordinates: 4 (256 x 128 181 against 164);
+//   linear kernel (three rings more): 4 (320 x 128 447 against 312), but for uniform sigma_T on
+//     193 .. 256 (175 against 207).
+int cells_per_lane(const SweepArgs &a, int n_items, int G, bool homog, int mom)
+{
+    const int I = a.I, sms = 152;
+    const bool inflow = a.inflow != nullptr, four = G == 4;
+    if (I <= 128 || n_items < 2 * sms) return 4;
+    if (mom == 0) return 8;  // (512 x 512 x 32 of 128: 1746 against 2054)
+    if (mom == 3) return homog && I > 192 && I <= 256 ? 8 : 4;
+    if ((I + 127) / 128 % 2 == 1) return homog && !four && n_items >= 4 * sms ? 8 : 4;
+    if (n_items < (inflow ? 4 : four ? 3 : 2) * sms) return 4;
+    if (!homog && four && (inflow || (I > 256 && (long long)n_items * a.J < 4000LL * sms)))
+        return 4;
+    return 8;
+}
 
 bool fits(int I, int mom, bool homog, int C)
 {
@@ -45,7 +69,7 @@ cudaError_t launch_sweep2d_ring(const SweepArgs &a, int n_items, int G, int sche
     if (!sweep2d_ring_fits(a.I, mom, homog) || (G != 1 && G != 2 && (G != 4 || mom == 0)) ||
         (a.grids != nullptr && (homog || a.inflow != nullptr || mom == 0)) || (!homog && a.gdesc == nullptr))
         return cudaErrorInvalidValue;
-    int C = cells_per_lane(a.I, n_items);
+    int C = cells_per_lane(a, n_items, G, homog, mom);
     if (!fits(a.I, mom, homog, C)) C = 8;  // wide rows: half the warps, the same rings
     if (mom == 0) return launch_sweep2d_ring_dense(a, n_items, C, G, scheme, homog, st);
     if (mom == 3)

@@ -596,25 +596,27 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
     };
 
     // x inflow, scaled, of rows r0 .. r0 + 7: lane e takes ordinate e % G of row r0 + e / G
+    // (32 is a multiple of G: the same ordinate in every pass)
     constexpr int kPre = (kGrp * G + 31) / 32;
-    float pre[kPre];
+    float pre[kPre], ix = 0.f, lw = 0.f;
+    const float *in = nullptr;
+    if (EDGE && w == 0 && A.inflow != nullptr) {
+#pragma unroll
+        for (int kk = 0; kk < G; ++kk)
+            if (kk == lane % G) {
+                if (kk < it.n) {
+                    ix = inj_x[kk];
+                    lw = A.ow[ord[kk]] * fabsf(A.oc[ord[kk]]) * gd.dy;
+                }
+                in = A.inflow + (long long)ord[kk] * A.inflow_stride + (XNEG ? J : 0);
+            }
+    }
     auto fetch = [&](int r0) {
 #pragma unroll
         for (int e = 0; e < kPre; ++e) {
-            const int k = (32 * e + lane) % G, rr = r0 + (32 * e + lane) / G;
-            float ix = 0.f, lw = 0.f;
-            long long o = 0;
-#pragma unroll
-            for (int kk = 0; kk < G; ++kk)
-                if (kk == k && kk < it.n) {
-                    ix = inj_x[kk];
-                    lw = A.ow[ord[kk]] * fabsf(A.oc[ord[kk]]) * gd.dy;
-                    o = ord[kk];
-                }
+            const int rr = r0 + (32 * e + lane) / G;
             float b = 0.f;
-            if (32 * e + lane < kGrp * G && rr >= 0 && rr < J)
-                b = A.inflow[(long long)o * A.inflow_stride + (XNEG ? J : 0) +
-                             (yneg ? J - 1 - rr : rr)];
+            if (32 * e + lane < kGrp * G && rr >= 0 && rr < J) b = in[yneg ? J - 1 - rr : rr];
             pre[e] = ix * b;
             leak -= (double)(lw * b);
         }

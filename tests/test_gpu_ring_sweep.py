@@ -142,3 +142,32 @@ def test_dense_mode(rom, grid, precision, medium, scheme, n_samples):
     ref, _ = oracle(I, J, st, ss, q, sets, inf, kernel="hg", g=0.4, scheme=scheme, fixed_iters=3)
     assert stats["rows_per_step"] == 1
     assert max(rel(phi[k], ref[k]) for k in range(n_samples)) < TOL
+
+
+@pytest.mark.parametrize("I,J,S,M,medium,tile_g,lit,kernel", [
+    (385, 21, 160, 9, "uniform", 2, False, "iso"),
+    (500, 13, 170, 9, "uniform", 4, False, "iso"),
+    (448, 21, 160, 9, "varying", 2, False, "iso"),
+    (391, 300, 512, 4, "varying", 4, False, "iso"),
+    (300, 13, 160, 9, "uniform", 2, False, "iso"),
+    (200, 21, 200, 9, "varying", 2, True, "iso"),
+    (131, 21, 200, 9, "varying", 4, True, "iso"),
+    (224, 17, 90, 9, "uniform", 2, False, "linear")])
+def test_lane_widths_of_large_batches(rom, I, J, S, M, medium, tile_g, lit, kernel):
+    """Batches on either side of the choice between 4 and 8 cells per lane (first, last and two
+    other samples against the oracle)."""
+    st, ss, q = W.random_medium(I, J, seed=I)
+    if medium == "uniform":
+        st = np.full((J, I), 2.1)
+        ss = np.minimum(ss, 1.8)
+    sets = [O.Ordinates(*W.random_directions(M, seed=50 + k, weights="random")) for k in range(S)]
+    inflow = np.random.default_rng(I).uniform(0.0, 1.5, 2 * J + 2 * I) if lit else None
+    phi, _, bal, stats = solve(rom, I, J, st, ss, q, sets, inflow, kernel=kernel, g=0.7,
+                               fixed_iters=2, tile_g=tile_g, rows_per_step=1)
+    some = [0, 1, S // 2, S - 1]
+    ref, _ = oracle(I, J, st, ss, q, [sets[k] for k in some], inflow, kernel=kernel, g=0.7,
+                    fixed_iters=2)
+    assert stats["rows_per_step"] == 1
+    for n, k in enumerate(some):
+        assert rel(phi[k], ref[n]) < TOL, k
+    assert np.all(bal < 1e-5)
