@@ -432,6 +432,13 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
 
     // One step.  EV: some lane passes its first or last row in this group of steps; ODD: P
     // holds its negative.
+    //
+    // Rows past the last one compute numbers that reach no cell of the grid: their source is what
+    // the lane left in the slot 16 rows before, and zero constants (k2, lx) keep them out of the
+    // y-edges and the leakage, as long as they are finite.  So such a row leaves nothing in its
+    // slot: one that took another's moments for a source would divide by sigma_T + a + b once
+    // more every 16 rows, and overflow in small units.  (Keeping P and lk by selects instead
+    // measured the same on most solves, 1-2% more on the smallest.)
     auto step = [&](auto events, auto odd) {
         constexpr bool EV = decltype(events)::value;
         constexpr bool ODD = DD && decltype(odd)::value;
@@ -559,7 +566,8 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
             for (int k = 0; k < MOM; ++k) v[k][r] = (!RAGGED || real[rr]) ? m[k].x + m[k].y : 0.f;
         }
 #pragma unroll
-        for (int k = 0; k < NS; ++k) sts_cells<C>(own, k * kArrB + slot, v[k], on);
+        for (int k = 0; k < NS; ++k)
+            sts_cells<C>(own, k * kArrB + slot, v[k], EV ? on && !past : on);
 #pragma unroll
         for (int q = 0; q < N; ++q) lk[q] = qfma(lx[q], x[C][q], lk[q]);
         if constexpr (MOM == 0) {
