@@ -259,9 +259,10 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
         qset(kms[pk], i, wm * s);
         qset(kc[pk], i, c);
         qset(ks[pk], i, s);
-        // leakage: w |s| dx y = (w dx dy / f) P; w |c| dy x = w |c| dy f rd X, or (w dx dy / f) X
-        qset(wl[pk], i, wt * gd.dx * gd.dy / fdd);
-        const float lo = HOMOG ? wt * fabsf(c) * gd.dy * fdd * rd : wt * gd.dx * gd.dy / fdd;
+        // leakage in units of dx dy, which can be outside the range of FP32 where the edge terms
+        // are not: w |s| dx y = dx dy (w / f) P; w |c| dy x = dx dy w a rd X, or dx dy (w / f) X
+        qset(wl[pk], i, wt / fdd);
+        const float lo = HOMOG ? wt * a * rd : wt / fdd;
         qset(lx[pk], i, (A.leak != nullptr && p == L - 1) ? lo : 0.f);
         inj_x[k] = HOMOG ? (st + a + b) / fdd : a;
         inj_y[k] = b;
@@ -614,7 +615,7 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
             if (kk == lane % G) {
                 if (kk < it.n) {
                     ix = inj_x[kk];
-                    lw = A.ow[ord[kk]] * fabsf(A.oc[ord[kk]]) * gd.dy;
+                    lw = A.ow[ord[kk]] * fabsf(A.oc[ord[kk]]) * gd.inv_dx;
                 }
                 in = A.inflow + (long long)ord[kk] * A.inflow_stride + (XNEG ? J : 0);
             }
@@ -686,7 +687,8 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
         leak += (double)(DD && ((J - 1 + lane) & 1) == 0 ? -lo : lo) + ((double)lk_s - (double)lk_c);
 #pragma unroll
         for (int dd = 16; dd > 0; dd >>= 1) leak += __shfl_xor_sync(0xffffffffu, leak, dd);
-        if (lane == 0 && leak != 0.0) atomicAdd(A.leak + it.sample, leak);
+        if (lane == 0 && leak != 0.0)
+            atomicAdd(A.leak + it.sample, leak * ((double)gd.dx * (double)gd.dy));
     }
 }
 

@@ -23,11 +23,12 @@ def rom():
 @pytest.mark.parametrize("kernel", ["iso", "linear"])
 @pytest.mark.parametrize("inflow", ["vacuum", "isotropic"])
 @pytest.mark.parametrize("tile_g", [2, 4])
-@pytest.mark.parametrize("unit", [1e-18])
+@pytest.mark.parametrize("unit", [1e-30, 1e-18, 1e22])
 def test_units_of_length(rom, scheme, medium, kernel, inflow, tile_g, unit):
     """Coefficients per length units other than the domain's own size.  1e-18: 1 / (sigma_T + a +
     b) is about 1e16, and a row that a lane computes past the grid's last one overflows if its
-    source is the moments of another such row.  None of it reaches the leakage or the balance."""
+    source is the moments of another such row.  None of it reaches the leakage or the balance.
+    1e-30 and 1e22: the area of a cell is outside the range of FP32, its edges are not."""
     I, J = 128, 21
     bounds = (0.0, 1.3 / unit, 0.0, 0.7 / unit)
     st, ss, q = (unit * a for a in W.random_medium(I, J, seed=5))
