@@ -351,10 +351,12 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
             if (held) k2[q] = k2n[q] = lx[q] = qsplat(0.f);
         }
     }
-    float lk_s = 0.f, lk_c = 0.f;  // compensated (Kahan) sum of the groups' x-edge terms
-    float2 lk[N];
+    // The x-edge terms, summed over the even and over the odd steps of a group, then compensated
+    // (Kahan): four rows per compensated add, as in the 4-row kernel.
+    float lk_s = 0.f, lk_c = 0.f;
+    float2 lk[2][N];
 #pragma unroll
-    for (int q = 0; q < N; ++q) lk[q] = qsplat(0.f);
+    for (int q = 0; q < N; ++q) lk[0][q] = lk[1][q] = qsplat(0.f);
 
     // Groups of 8 steps of the warp: steps -8 .. J + 7 + 8 * (its last lanes' group); a warp
     // starts kLag groups after the one upstream.  nwl: warps that own cells (a batch's
@@ -442,7 +444,8 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
     // measured the same on most solves, 1-2% more on the smallest.)
     auto step = [&](auto events, auto odd) {
         constexpr bool EV = decltype(events)::value;
-        constexpr bool ODD = DD && decltype(odd)::value;
+        constexpr int par = decltype(odd)::value;
+        constexpr bool ODD = DD && par;
         fill();
         // the moments of the row that the group's last lane finished at the step before
         // (fill has moved on to its slot)
@@ -570,7 +573,7 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
         for (int k = 0; k < NS; ++k)
             sts_cells<C>(own, k * kArrB + slot, v[k], EV ? on && !past : on);
 #pragma unroll
-        for (int q = 0; q < N; ++q) lk[q] = qfma(lx[q], x[C][q], lk[q]);
+        for (int q = 0; q < N; ++q) lk[par][q] = qfma(lx[q], x[C][q], lk[par][q]);
         if constexpr (MOM == 0) {
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
@@ -665,13 +668,16 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
                     step(std::false_type{}, std::true_type{});
                 }
             }
-            const float yv = (N == 2 ? (lk[0].x + lk[0].y) + (lk[N - 1].x + lk[N - 1].y)
-                                     : lk[0].x + lk[0].y) - lk_c;
-            const float tt = lk_s + yv;
-            lk_c = (tt - lk_s) - yv;
-            lk_s = tt;
 #pragma unroll
-            for (int q = 0; q < N; ++q) lk[q] = qsplat(0.f);
+            for (int h = 0; h < 2; ++h) {
+                const float2 &l0 = lk[h][0], &l1 = lk[h][N - 1];
+                const float yv = (N == 2 ? (l0.x + l0.y) + (l1.x + l1.y) : l0.x + l0.y) - lk_c;
+                const float tt = lk_s + yv;
+                lk_c = (tt - lk_s) - yv;
+                lk_s = tt;
+#pragma unroll
+                for (int q = 0; q < N; ++q) lk[h][q] = qsplat(0.f);
+            }
         }
         if (EDGE && nw > 1) __syncthreads();
     }

@@ -59,3 +59,30 @@ def test_units_of_length(rom, scheme, medium, kernel, inflow, tile_g, unit):
         scale = abs(ref["leak"][k]) + np.sum(st * ref["phi"][k]) * area
         assert abs(leak[k] - ref["leak"][k]) < 1e-5 * scale
     assert np.all(bal < 1e-5) and np.isfinite(stats["balance_max"])
+
+
+@pytest.mark.parametrize("scheme", ["dd", "step"])
+@pytest.mark.parametrize("medium", ["uniform", "varying"])
+@pytest.mark.parametrize("tile_g", [2, 4])
+def test_rows_per_compensated_add(rom, scheme, medium, tile_g):
+    """The x-face terms of the leakage go into the compensated sum at most four rows at a time.
+    One ordinate along x, eight rows in one lane; the first carries 1, the others 2^-26, which
+    an FP32 sum with the first's term drops (at most a quarter of its last place).  Of the seven,
+    the four outside the first's sum stay: at least half of what they let out."""
+    I, J, small = 4, 8, 2.0 ** -26
+    st = np.full((J, I), 1e-3)
+    if medium == "varying":
+        st[0, 0] = 1.5e-3
+    leak = []
+    for rest in (0.0, small):
+        ctx = rom.RomContext(0)
+        ctx.set_grid(I, J, (0.0, 1.0, 0.0, float(J)), st, 0.0 * st, 0.0 * st)
+        ctx.set_ordinates([(np.array([1.0]), np.array([0.0]), np.array([0.0]), np.array([1.0]))])
+        ctx.set_inflow_isotropic(0, np.array([1.0] + [rest] * (J - 1)))
+        ctx.set_options(scheme=rom.SCHEME[scheme], fixed_iters=1, tile_g=tile_g, rows_per_step=1)
+        ctx.solve()
+        leak.append(float(ctx.balance()[0][0]))
+        ctx.close()
+    # leakage = what goes out less what comes in; dy = 1, and e^-0.001 of the inflow passes
+    out = (leak[1] - leak[0]) + 7 * small
+    assert 0.5 * 7 * small * 0.99 < out < 1.01 * 7 * small
