@@ -1,5 +1,6 @@
 // sweep2d_row.cu -- the one-row-per-step X-Y sweep kernels (sweep2d_row.cuh) for
-// one grid: the diamond-difference isotropic moment mode here, and the dispatch
+// one grid: the diamond-difference isotropic moment mode here (sigma_T varying;
+// with one sigma_T every row runs on the rings of sweep2d_ring.cuh), and the dispatch
 // to the other translation units (sweep2d_row_step.cu: step scheme;
 // sweep2d_row_m3.cu: linear-kernel moments; sweep2d_row_dense.cu: the dense
 // operator mode; sweep2d_row_batch.cu: batches of several grids), which build in

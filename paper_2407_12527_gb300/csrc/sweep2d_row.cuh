@@ -544,8 +544,9 @@ __global__ void __launch_bounds__(32 * kMaxWarps) sweep2d_row_kernel(const Sweep
 }
 
 // one kernel per (G, homog, inflow) of this translation unit's source
-// mode MOM and scheme SCHEME; items of one ordinate run on the two-ordinate
-// kernel (the empty second slot has zero weight)
+// mode MOM and scheme SCHEME that a row can need (the rings of sweep2d_ring.cuh
+// come first); items of one ordinate run on the two-ordinate kernel (the empty
+// second slot has zero weight)
 template <int MOM, int SCHEME, bool BATCH>
 cudaError_t row_launch(const SweepArgs &a, int n_items, int nwarps, int G, bool homog,
                        cudaStream_t st)
@@ -565,6 +566,11 @@ cudaError_t row_launch(const SweepArgs &a, int n_items, int nwarps, int G, bool 
         (void)homog;  // several grids: sigma_T read per cell, vacuum boundaries
         if (G == 4) ROW_K(4, false, false);
         else ROW_K(2, false, false);
+    } else if constexpr (MOM == 1) {
+        // one sigma_T: the rings of the widest row (2048 cells, 8 warps, 132 KB) fit a CTA
+        if (homog) return cudaErrorInvalidValue;
+        if (G == 4) ROW_G(4, false);
+        else ROW_G(2, false);
     } else {
         if constexpr (MOM != 0) {  // (the dense mode takes at most two ordinates per item)
             if (G == 4) {

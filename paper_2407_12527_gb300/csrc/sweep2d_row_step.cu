@@ -1,5 +1,5 @@
 // sweep2d_row_step.cu -- the one-row-per-step X-Y sweep (sweep2d_row.cuh) for one
-// grid, step scheme, isotropic moment mode.
+// grid, step scheme, isotropic moment mode (sigma_T varying).
 #include "sweep2d_row.cuh"
 
 namespace romk {
