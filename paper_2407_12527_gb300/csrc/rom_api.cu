@@ -897,7 +897,7 @@ cudaError_t launch_xy_sweep(const rom_ctx *ctx, const romk::SweepArgs &sa, int G
     const int nwarps = (L + 31) / 32;
     if (H == 1 && ring_sweep(ctx))
         return romk::launch_sweep2d_ring(sa, (int)ctx->items.size(), G, ctx->opt.scheme,
-                                         ctx->homog && !batch(ctx), ctx->MOM, st);
+                                         ctx->homog && !batch(ctx), ctx->MOM, ctx->sm_count, st);
     if (H == 1) {
         if (batch(ctx))
             return romk::launch_sweep2d_row_batch(sa, (int)ctx->items.size(), nwarps, G,

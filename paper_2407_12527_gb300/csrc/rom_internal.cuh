@@ -352,7 +352,7 @@ cudaError_t launch_sweep2d_row_batch(const SweepArgs &a, int n_items, int nwarps
 // or a batch of them (a.I: the widest); fits: whether a row's rings fit a CTA
 bool sweep2d_ring_fits(int I, int mom, bool homog);
 cudaError_t launch_sweep2d_ring(const SweepArgs &a, int n_items, int G, int scheme, bool homog,
-                                int mom, cudaStream_t st);
+                                int mom, int sm_count, cudaStream_t st);
 cudaError_t launch_sweep3d(const Sweep3Args &a, int n_ctas, int nwarps, int G, int scheme,
                            cudaStream_t st);
 int sweep3d_ctas_per_sm(int nwarps, int G);

@@ -35,9 +35,9 @@ namespace {
 //   inflow with varying sigma_T and four ordinates: 4 (256 x 128 181 against 164);
 //   linear kernel (three rings more): 4 (320 x 128 447 against 312), but for uniform sigma_T on
 //     193 .. 256 (175 against 207).
-int cells_per_lane(const SweepArgs &a, int n_items, int G, bool homog, int mom)
+int cells_per_lane(const SweepArgs &a, int n_items, int G, bool homog, int mom, int sms)
 {
-    const int I = a.I, sms = 152;
+    const int I = a.I;
     const bool inflow = a.inflow != nullptr, four = G == 4;
     if (I <= 128 || n_items < 2 * sms) return 4;
     if (mom == 0) return 8;  // (512 x 512 x 32 of 128: 1746 against 2054)
@@ -63,13 +63,13 @@ bool sweep2d_ring_fits(int I, int mom, bool homog)
 }
 
 cudaError_t launch_sweep2d_ring(const SweepArgs &a, int n_items, int G, int scheme, bool homog,
-                                int mom, cudaStream_t st)
+                                int mom, int sm_count, cudaStream_t st)
 {
     if (n_items <= 0) return cudaSuccess;
     if (!sweep2d_ring_fits(a.I, mom, homog) || (G != 1 && G != 2 && (G != 4 || mom == 0)) ||
         (a.grids != nullptr && (homog || a.inflow != nullptr || mom == 0)) || (!homog && a.gdesc == nullptr))
         return cudaErrorInvalidValue;
-    int C = cells_per_lane(a, n_items, G, homog, mom);
+    int C = cells_per_lane(a, n_items, G, homog, mom, sm_count);
     if (!fits(a.I, mom, homog, C)) C = 8;  // wide rows: half the warps, the same rings
     if (mom == 0) return launch_sweep2d_ring_dense(a, n_items, C, G, scheme, homog, st);
     if (mom == 3)
