@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(256) combine_kernel(const CombineArgs A0)
         base = A0.soff[s];
     }
     const long long cells = A.cells;  // a multiple of 8: a thread takes whole 32-byte sectors
-    float *phi = A.phi + base;
+    float *phi = A.phi + base / MOM;
     float *src = A.src + base;
     float d2f = 0.f, n2f = 0.f, mn = INFINITY, a1f = 0.f, b0f = 0.f, b1f = 0.f, b2f = 0.f;
     // KS sectors per thread and pass, all loaded before any store (the loads and
@@ -375,14 +375,15 @@ __global__ void init_state_kernel(int S, int MOM, long long cells, const float *
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
     const long long n4 = cells / 4;  // (cells is a multiple of 8)
     for (long long sm = blockIdx.y; sm < (long long)S * MOM; sm += gridDim.y) {
-        float4 *p = (float4 *)(phi + sm * cells), *a = (float4 *)(part + sm * cells);
+        float4 *p = (float4 *)(phi + sm / MOM * cells), *a = (float4 *)(part + sm * cells);
         float4 *f = (float4 *)(src + sm * cells);
+        const bool first = sm % MOM == 0;
         for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n4;
              v += (long long)gridDim.x * blockDim.x) {
-            p[v] = zero;
+            if (first) p[v] = zero;
             if (part) a[v] = zero;
             // psi^0 = 0: the first source is q
-            if (src) f[v] = sm % MOM == 0 ? ((const float4 *)q)[v] : zero;
+            if (src) f[v] = first ? ((const float4 *)q)[v] : zero;
         }
     }
     if (blockIdx.y > 0) return;
@@ -417,12 +418,12 @@ __global__ void init_grids_kernel(int MOM, const GridDesc *grids, const int *sgr
     for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n;
          v += (long long)gridDim.x * blockDim.x) {
         const long long cell = v % g.cells;
-        phi[soff[s] + v] = 0.f;
+        if (v < g.cells) phi[soff[s] / MOM + v] = 0.f;
         src[soff[s] + v] = v < g.cells ? q[g.off + cell] : 0.f;
     }
 }
 
-__global__ void average_kernel(const float *phi, int S, int MOM, int I, int J, int NXP,
+__global__ void average_kernel(const float *phi, int S, int I, int J, int NXP,
                                double *avg, double *sum)
 {
     const long long cells = (long long)J * NXP;
@@ -431,18 +432,17 @@ __global__ void average_kernel(const float *phi, int S, int MOM, int I, int J, i
          v += (long long)gridDim.x * blockDim.x) {
         const long long j = v / I, i = v - j * I;
         double acc = 0.0;
-        for (int s = 0; s < S; ++s) acc += (double)phi[(long long)s * MOM * cells + j * NXP + i];
+        for (int s = 0; s < S; ++s) acc += (double)phi[(long long)s * cells + j * NXP + i];
         if (sum) sum[v] = acc;
         if (avg) avg[v] = S > 0 ? acc / S : 0.0;
     }
 }
 
-__global__ void extract_kernel(const float *phi, int sample, int MOM, int I, int J, int NXP,
-                               double *out)
+__global__ void extract_kernel(const float *phi, int sample, int I, int J, int NXP, double *out)
 {
     const long long cells = (long long)J * NXP;
     const long long n = (long long)I * J;
-    const float *p = phi + (long long)sample * MOM * cells;
+    const float *p = phi + (long long)sample * cells;
     for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n;
          v += (long long)gridDim.x * blockDim.x) {
         const long long j = v / I, i = v - j * I;
@@ -569,18 +569,18 @@ cudaError_t launch_init_grids(int S, int MOM, const GridDesc *grids, const int *
     return cudaGetLastError();
 }
 
-cudaError_t launch_average(const float *phi, int S, int MOM, int I, int J, int NXP, double *avg,
+cudaError_t launch_average(const float *phi, int S, int I, int J, int NXP, double *avg,
                            double *sum, cudaStream_t st)
 {
-    average_kernel<<<blocks_for((long long)I * J, 256), 256, 0, st>>>(phi, S, MOM, I, J, NXP, avg,
+    average_kernel<<<blocks_for((long long)I * J, 256), 256, 0, st>>>(phi, S, I, J, NXP, avg,
                                                                        sum);
     return cudaGetLastError();
 }
 
-cudaError_t launch_extract(const float *phi, int sample, int MOM, int I, int J, int NXP,
-                           double *out, cudaStream_t st)
+cudaError_t launch_extract(const float *phi, int sample, int I, int J, int NXP, double *out,
+                           cudaStream_t st)
 {
-    extract_kernel<<<blocks_for((long long)I * J, 256), 256, 0, st>>>(phi, sample, MOM, I, J, NXP,
+    extract_kernel<<<blocks_for((long long)I * J, 256), 256, 0, st>>>(phi, sample, I, J, NXP,
                                                                        out);
     return cudaGetLastError();
 }

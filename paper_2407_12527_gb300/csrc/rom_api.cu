@@ -1106,10 +1106,10 @@ int ensure_state(rom_ctx *ctx)
             return rc;
         return ROM_OK;
     }
-    // [S][MOM][J][NXP], or each sample's [MOM][J_p][NXP_p] block of its grid
+    // [S][MOM][J][NXP], or each sample's [MOM][J_p][NXP_p] block of its grid; phi one moment
     const size_t b = (batch(ctx) ? (size_t)ctx->state_floats
                                  : S * MOM * (size_t)padded_cells(ctx)) * sizeof(float);
-    if ((rc = ensure(ctx, ctx->phi, b)) || (rc = ensure(ctx, ctx->src, b)) ||
+    if ((rc = ensure(ctx, ctx->phi, b / MOM)) || (rc = ensure(ctx, ctx->src, b)) ||
         (rc = ensure(ctx, ctx->part, b)))
         return rc;
     return ROM_OK;
@@ -2007,19 +2007,19 @@ int rom_solve(rom_ctx *ctx, rom_stats *stats_out)
         CK(romk::launch_average3((const float *)ctx->phi.p, ctx->S,
                                  romk::make_skew3(ctx->J, ctx->K, ctx->NXP), ctx->I,
                                  (double *)ctx->avg.p, (double *)ctx->sum.p, ctx->stream));
-    else if (batch(ctx)) {  // each grid's samples are consecutive [MOM][J_p][NXP_p] blocks
+    else if (batch(ctx)) {  // each grid's samples are consecutive [J_p][NXP_p] blocks
         int s0 = 0;
         for (int p = 0; p < ctx->n_grids; ++p) {
             const romk::GridDesc &g = ctx->grids[p];
-            CK(romk::launch_average((const float *)ctx->phi.p + ctx->soff[s0],
-                                    ctx->grid_samples[p], MOM, g.I, g.J, g.NXP,
+            CK(romk::launch_average((const float *)ctx->phi.p + ctx->soff[s0] / MOM,
+                                    ctx->grid_samples[p], g.I, g.J, g.NXP,
                                     (double *)ctx->avg.p + ctx->avg_off[p],
                                     (double *)ctx->sum.p + ctx->avg_off[p], ctx->stream));
             s0 += ctx->grid_samples[p];
         }
         ctx->launches += ctx->n_grids - 1;
     } else
-        CK(romk::launch_average((const float *)ctx->phi.p, ctx->S, MOM, ctx->I, (int)ctx->rows,
+        CK(romk::launch_average((const float *)ctx->phi.p, ctx->S, ctx->I, (int)ctx->rows,
                                 ctx->NXP, (double *)ctx->avg.p, (double *)ctx->sum.p,
                                 ctx->stream));
     ++ctx->launches;
@@ -2102,16 +2102,15 @@ cudaError_t extract_phi(rom_ctx *ctx, int sample, double *out)
 {
     if (batch(ctx)) {
         const romk::GridDesc &g = ctx->grids[ctx->sgrid[sample]];
-        return romk::launch_extract((const float *)ctx->phi.p + ctx->soff[sample], 0,
-                                    ctx->MOM == 0 ? 1 : ctx->MOM, g.I, g.J, g.NXP, out,
-                                    ctx->stream);
+        return romk::launch_extract((const float *)ctx->phi.p + ctx->soff[sample] / ctx->MOM, 0,
+                                    g.I, g.J, g.NXP, out, ctx->stream);
     }
     if (ctx->dim == 3)
         return romk::launch_extract3((const float *)ctx->phi.p, sample,
                                      romk::make_skew3(ctx->J, ctx->K, ctx->NXP), ctx->I, out,
                                      ctx->stream);
-    return romk::launch_extract((const float *)ctx->phi.p, sample, ctx->MOM == 0 ? 1 : ctx->MOM,
-                                ctx->I, (int)ctx->rows, ctx->NXP, out, ctx->stream);
+    return romk::launch_extract((const float *)ctx->phi.p, sample, ctx->I, (int)ctx->rows, ctx->NXP,
+                                out, ctx->stream);
 }
 
 int rom_get_scalar_flux(rom_ctx *ctx, int sample, double *out)

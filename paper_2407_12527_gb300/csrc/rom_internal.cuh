@@ -4,12 +4,13 @@
 // HBM layout (all FP32 unless noted; rows padded to a pitch of NXP = ceil(I/8)*8
 // floats so every lane's 8-cell segment is one aligned 32-byte sector):
 //   sigma_t, sigma_s, q      [J][NXP]
-//   phi    (per sample)      [S][MOM][J][NXP]   current iterate, MOM scalar moments
+//   phi    (per sample)      [S][J][NXP]        current iterate (scalar flux)
 //   src    (per sample)      [S][MOM][J][NXP]   source moments for the next sweep
 //   part   (per sample)      [S][MOM][J][NXP]   moments the sweep's work items add
 //   ordinates                c, s, w [M_total] (FP32) and c, s, zeta, w (FP64)
 //   residual and balance sums [S][kNP] FP64, smallest phi [S] (ordered-int key)
-// MOM = 1 for isotropic scattering (phi), 3 for the linear kernel (phi, Jx, Jy).
+// MOM = 1 for isotropic scattering (phi), 3 for the linear kernel (phi, Jx, Jy; the currents
+// of an iterate are kept only in the source they enter).
 // 3D grids keep the arrays their sweep touches in diagonal storage (Skew3 below).
 #pragma once
 
@@ -99,7 +100,7 @@ struct CombineArgs {
     long long cells;
     float g;                    // linear-kernel asymmetry (MOM = 3)
     float *acc;                 // [S][MOM][cells] moments added by the sweep, cleared here
-    float *phi;
+    float *phi;                 // [S][cells]
     float *src;
     const float *sigma_s, *q;
     // balance sums (moment modes): sigma_T per cell, nullptr = sigma_t_homog
@@ -109,7 +110,7 @@ struct CombineArgs {
     // several grids (nullptr: one): the sample's grid and state offset
     const GridDesc *grids;
     const int *sgrid;           // [S]
-    const long long *soff;      // [S]
+    const long long *soff;      // [S] (of phi: divided by MOM)
     const int *active;
     double *sums;               // [S][kNP] added with FP64 atomics
     int *minkey;                // [S] smallest phi (float_order_key), atomic min
@@ -393,18 +394,18 @@ struct InitState {
     int *minkey;
     unsigned long long *going;
 };
-// the same launch sets phi = 0, the first source (q; nullptr: kept elsewhere) and the
-// cleared accumulators part (nullptr: not here) of [S][MOM][cells] values
+// the same launch sets phi [S][cells] = 0, and in arrays of [S][MOM][cells] values the first
+// source (q; nullptr: kept elsewhere) and the cleared accumulators part (nullptr: not here)
 cudaError_t launch_init_state(int S, int MOM, long long cells, const float *q, float *phi,
                               float *src, float *part, const InitState &is, cudaStream_t st);
-cudaError_t launch_average(const float *phi, int S, int MOM, int I, int J, int NXP, double *avg,
+cudaError_t launch_average(const float *phi, int S, int I, int J, int NXP, double *avg,
                            double *sum, cudaStream_t st);
 // several grids: phi = 0 and the first source q for every sample on its own grid
 cudaError_t launch_init_grids(int S, int MOM, const GridDesc *grids, const int *sgrid,
                               const long long *soff, int max_cells, const float *q, float *phi,
                               float *src, cudaStream_t st);
-cudaError_t launch_extract(const float *phi, int sample, int MOM, int I, int J, int NXP,
-                           double *out, cudaStream_t st);
+cudaError_t launch_extract(const float *phi, int sample, int I, int J, int NXP, double *out,
+                           cudaStream_t st);
 cudaError_t launch_pad_grid(const float *st_in, const float *ss_in, const float *q_in, int I,
                             int J, int NXP, float *st_out, float *ss_out, float *q_out,
                             unsigned int *stats /*[3]: min sigma_t bits, max bits, bad cells*/,
