@@ -33,7 +33,10 @@
 //   varying sigma_T: X = a x, P = b y: psi = (S + X + P) / d, X' = f a psi - X (DD) or
 //     a psi, P' likewise, moment += w psi.
 // The uniform case takes five packed FP32x2 operations per cell and ordinate pair and its
-// upwind chain is one FMA per cell.  The DD closure keeps -P after even steps (and the
+// upwind chain is one FMA per cell.  (DD in uniform cells of many mean free paths: X and X'
+// nearly cancel, and their sum has the rounding of the edges instead of psi's.  The 4-row
+// kernel's x + x' is the same: over twelve lit media without sources the flux is off by
+// 8e-7 on average at sigma_T dx = 100 and 6e-6 at 1000 with either.)  The DD closure keeps -P after even steps (and the
 // varying case -X at odd cells), so that every update is one FMA without a negated operand:
 // P' = c - P or -P' = P - c.  (Negated operands cost the packed instructions nothing; the
 // plain form measured 4% slower on the checkerboard with four ordinates per item, 7% faster
@@ -352,11 +355,10 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
         }
     }
     // The x-edge terms, summed over the even and over the odd steps of a group, then compensated
-    // (Kahan): four rows per compensated add, as in the 4-row kernel.
+    // (Kahan): four rows of the item's pairs per compensated add, as in the 4-row kernel.  (A sum
+    // per pair has registers spilled with four ordinates: 0.5% slower over 33 solves.)
     float lk_s = 0.f, lk_c = 0.f;
-    float2 lk[2][N];
-#pragma unroll
-    for (int q = 0; q < N; ++q) lk[0][q] = lk[1][q] = qsplat(0.f);
+    float2 lk[2] = {qsplat(0.f), qsplat(0.f)};
 
     // Groups of 8 steps of the warp: steps -8 .. J + 7 + 8 * (its last lanes' group); a warp
     // starts kLag groups after the one upstream.  nwl: warps that own cells (a batch's
@@ -573,7 +575,7 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
         for (int k = 0; k < NS; ++k)
             sts_cells<C>(own, k * kArrB + slot, v[k], EV ? on && !past : on);
 #pragma unroll
-        for (int q = 0; q < N; ++q) lk[par][q] = qfma(lx[q], x[C][q], lk[par][q]);
+        for (int q = 0; q < N; ++q) lk[par] = qfma(lx[q], x[C][q], lk[par]);
         if constexpr (MOM == 0) {
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
@@ -670,13 +672,11 @@ __device__ __forceinline__ void ring_item(const SweepArgs &A, const GridDesc &gd
             }
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const float2 &l0 = lk[h][0], &l1 = lk[h][N - 1];
-                const float yv = (N == 2 ? (l0.x + l0.y) + (l1.x + l1.y) : l0.x + l0.y) - lk_c;
+                const float yv = (lk[h].x + lk[h].y) - lk_c;
                 const float tt = lk_s + yv;
                 lk_c = (tt - lk_s) - yv;
                 lk_s = tt;
-#pragma unroll
-                for (int q = 0; q < N; ++q) lk[h][q] = qsplat(0.f);
+                lk[h] = qsplat(0.f);
             }
         }
         if (EDGE && nw > 1) __syncthreads();
@@ -704,9 +704,7 @@ __global__ void __launch_bounds__(MAXT) sweep2d_ring_kernel(const SweepArgs A)
     extern __shared__ __align__(1024) char ring_smem[];
     const SweepItem it = A.items[blockIdx.x];
     if (!A.active[it.sample]) return;
-    // Several grids vary in sigma_T: those kernels take every grid from the table, one grid
-    // too (a choice here between the table and the arguments' fields was miscompiled: the
-    // width alone stayed the arguments').
+    // sigma_T varying: the grid from the table, whether it holds one or several
     GridDesc gd{A.I, A.J, A.NXP, A.inv_dx, A.inv_dy, A.dx, A.dy, 0, A.cells};
     if constexpr (!HOMOG) gd = A.gdesc[it.grid];
     if (A.stall) {  // test hook: every warp waits on a barrier that nothing completes
