@@ -349,8 +349,8 @@ cudaError_t launch_sweep2d_row(const SweepArgs &a, int n_items, int nwarps, int 
                                bool homog, int mom, cudaStream_t st);
 cudaError_t launch_sweep2d_row_batch(const SweepArgs &a, int n_items, int nwarps, int G,
                                      int scheme, int mom, cudaStream_t st);
-// the moment modes with the rows staged through shared memory (sweep2d_ring.cuh), one grid
-// or a batch of them (a.I: the widest); fits: whether a row's rings fit a CTA
+// the same with the rows staged through shared memory (sweep2d_ring.cuh), one grid or, in the
+// moment modes, a batch of them (a.I: the widest); fits: whether a row's rings fit a CTA
 bool sweep2d_ring_fits(int I, int mom, bool homog);
 cudaError_t launch_sweep2d_ring(const SweepArgs &a, int n_items, int G, int scheme, bool homog,
                                 int mom, int sm_count, cudaStream_t st);

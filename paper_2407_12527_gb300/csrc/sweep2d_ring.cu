@@ -24,23 +24,26 @@ namespace {
 // width to 128 cells instead of 256.  Microseconds per sweep, 8 against 4 cells, samples of 16:
 //   up to 256 wide: 8, unless there are too few items to share the schedulers (2 per SM, of
 //     four ordinates 3, with inflow 4: 256 x 256, 1200 items of two 89 against 126, 128 of two
-//     43 against 35; 600 of four 64 against 80; three grids up to 200 wide, 384 of four 108
-//     against 74; 211 x 173 with inflow, varying sigma_T, 384 of two 87 against 73);
+//     43 against 39; 600 of four 65 against 80; three grids up to 200 wide, 384 of four 94
+//     against 64; 211 x 173 with inflow, varying sigma_T, 384 of two 76 against 66);
 //   257 .. 384 (more generally where 256-cell warps round up further): 4 (320 x 256, varying
-//     sigma_T, 600 of four 261 against 145), but for uniform sigma_T with two ordinates (147
-//     against 176);
-//   above: 8 (512 x 256 uniform 184 against 250), but for varying sigma_T with four ordinates,
-//     whose 220 registers and 64 KB of rings want many long items (448 x 64, 2000 items 395
-//     against 319; 448 x 448, 2048 of uneven samples 945 against 1000);
-//   inflow with varying sigma_T and four ordinates: 4 (256 x 128 181 against 164);
-//   linear kernel (three rings more): 4 (320 x 128 447 against 312), but for uniform sigma_T on
-//     193 .. 256 (175 against 207).
+//     sigma_T, 600 of four 221 against 147), but for uniform sigma_T with two ordinates (1200
+//     of two 151 against 175);
+//   above: 8 (512 x 256 uniform, 1200 of two 187 against 246), but for varying sigma_T with four
+//     ordinates, whose 212 registers and 64 KB of rings want many items (448 x 64, 600 items 118
+//     against 107; 448 x 448, 2048 of uneven samples 946 against 1098; the line is that of an
+//     earlier form of the kernel, the present one gains from about 2000 items on, 448 x 64 306
+//     against 326);
+//   inflow with varying sigma_T and four ordinates: 4 (1200 items on 448 x 128 316 against 289,
+//     on 144 x 128 141 against 138, but on 256 x 128 156 against 165);
+//   linear kernel (three rings more): 4 (320 x 128, 1200 of four 440 against 305), but for
+//     uniform sigma_T on 193 .. 256 (256 x 128 172 against 205).
 int cells_per_lane(const SweepArgs &a, int n_items, int G, bool homog, int mom, int sms)
 {
     const int I = a.I;
     const bool inflow = a.inflow != nullptr, four = G == 4;
     if (I <= 128 || n_items < 2 * sms) return 4;
-    if (mom == 0) return 8;  // (512 x 512 x 32 of 128: 1746 against 2054)
+    if (mom == 0) return 8;  // (512 x 512 x 32 of 128: 1750 against 2136)
     if (mom == 3) return homog && I > 192 && I <= 256 ? 8 : 4;
     if ((I + 127) / 128 % 2 == 1) return homog && !four && n_items >= 4 * sms ? 8 : 4;
     if (n_items < (inflow ? 4 : four ? 3 : 2) * sms) return 4;
