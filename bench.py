@@ -38,6 +38,8 @@ METRIC = "cell-ordinate updates/s (ROM source iteration, 1 GB300)"
 UNIT = "updates/s"
 FLOP_PER_UPDATE = 11  # diamond difference, homogeneous sigma_T: 5 FMA + 1 MUL
 FLOP_PER_UPDATE_HET = 13  # heterogeneous sigma_T: + 1 add + 1 reciprocal per cell-ordinate
+# the ring sweep and the choice of its instance (cells per lane)
+RING_SOURCES = "sweep2d_ring.cuh sweep2d_ring.cu"
 FLOP_PER_UPDATE_RING = 8       # one-row sweep: 2 ADD + 3 FMA in scaled edge fluxes
 FLOP_PER_UPDATE_RING_HET = 11  # varying sigma_T: 3 ADD + reciprocal + MUL + 3 FMA
 FLOP_PER_UPDATE_3D = 17   # 3D, heterogeneous: 3 FMA + add + reciprocal + MUL, 3 FMA outflows, 1 FMA phi
@@ -192,10 +194,11 @@ class ClockSampler:
 def traffic_record(name, source_file, samples_now, shape=None):
     """DRAM bytes of one full launch (every sample active) of a kernel, from the
     committed ncu capture profiles/<name>.traffic.json, scaled from the captured
-    batch to samples_now samples; None when the kernel source differs from the
-    one captured (sha256) or no record exists.  Records with a "shapes" table
-    hold one capture per work-item shape (e.g. "G2H1": 2 ordinates per item, one
-    row per step), each with the source file it was built from."""
+    batch to samples_now samples; None when the kernel source (one file, or
+    several separated by blanks: the sha256 is of all of them in that order)
+    differs from the one captured or no record exists.  Records with a "shapes"
+    table hold one capture per work-item shape (e.g. "G2H1": 2 ordinates per item,
+    one row per step), each with the source it was built from."""
     import hashlib
     tpath = os.path.join(ROOT, "profiles", name + ".traffic.json")
     if not os.path.exists(tpath):
@@ -211,10 +214,11 @@ def traffic_record(name, source_file, samples_now, shape=None):
         rec = tr
     if source_file is None:
         return None
-    spath = os.path.join(ROOT, "paper_2407_12527_gb300", "csrc", source_file)
-    with open(spath, "rb") as f:
-        digest = hashlib.sha256(f.read()).hexdigest()
-    if rec.get("source_sha256") != digest:
+    digest = hashlib.sha256()
+    for part in source_file.split():
+        with open(os.path.join(ROOT, "paper_2407_12527_gb300", "csrc", part), "rb") as f:
+            digest.update(f.read())
+    if rec.get("source_sha256") != digest.hexdigest():
         return None
     return rec["dram_bytes_per_launch"] * samples_now / tr["samples"]
 
@@ -492,7 +496,7 @@ def run_ours(args):
     elif WL.name == "lognormal_cube" and s["tile_g"] == 2:
         traffic = traffic_record("sweep3d_lognormal_cube_128", "sweep3d.cu", WL.samples)
     elif WL.name == "checkerboard" and s["tile_g"] == 4 and s["rows_per_step"] == 1:
-        traffic = traffic_record("sweep2d_checkerboard_448", "sweep2d_ring.cuh", WL.samples)
+        traffic = traffic_record("sweep2d_checkerboard_448", RING_SOURCES, WL.samples)
     if tc and src_ms > 0:
         roofline = {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                     "frac": achieved / hbm_peak,
@@ -514,7 +518,7 @@ def run_ours(args):
             roofline = {"bound": "hbm", "achieved": sw, "peak": hbm_peak, "unit": "GB/s",
                         "frac": sw / hbm_peak,
                         "traffic": traffic_record("sweep2d_dense_hg_disc_512",
-                                                  "sweep2d_ring.cuh", WL.samples),
+                                                  RING_SOURCES, WL.samples),
                         "traffic_note": "DRAM read+write bytes of one launch with every sample "
                                         "active (ncu, scaled by samples); achieved counts the "
                                         "algorithmic bytes, 8 B per cell-ordinate update",
